@@ -799,7 +799,7 @@ extern "C" vpm_status vpm_induce_noalloc(const float* src_pos_d, const float* sr
             "src_pos/src_str must be 16-byte aligned device pointers");
     const bool comp = flags & VPM_COMPENSATED;
     Carve cv;
-    const SweepPlan p = plan_sweep(n_tgt, n_src, 0, grad_u_d != nullptr, comp, cv);
+    const SweepPlan p = plan_sweep(n_tgt, n_src, 0, grad_u_d != nullptr, comp, cv, false, false);
     if (!overflow_guard(p)) return fail(VPM_ERR_LIMIT, "problem too large for the stream-K split");
     if (p.bytes > (size_t)VPM_NOALLOC_SCRATCH_BYTES)
         return fail(VPM_ERR_LIMIT,

@@ -1,0 +1,153 @@
+// Far-field part of the particle sweep on the 5th-generation tensor cores.
+//
+// A source tile (128 consecutive particles) seen from far away is a contraction: with
+// c the tile's centre, a its scale, d_j = (x_j - c)/a, and for a target y = x - c,
+// n = y/|y|, e = a/|y|, the separation is r = |y| (n - e d_j) and every pair's kernels are
+//   r^-5 = |y|^-5 t^(-5/2),  r^-3 = |y|^-5 t^(-5/2) r^2,   t = 1 - 2 e n.d_j + e^2 |d_j|^2.
+// u and grad u are then fixed combinations (polynomials in n and e) of the sums
+//   m_f = sum_j t_j^(-5/2) F_f(j)
+// over 29 source features F (Gamma, Gamma x d, their products with d, |d|^2): a matrix
+// product [targets x sources] [sources x features].  Every pair's t^(-5/2) is evaluated
+// (7 FP32 operations and one rsqrt against 32 and one in the pair loop); the product runs
+// on tcgen05 with the targets in the rows of a TMEM operand.
+//
+// Precision.  m_f is split as sum_j F_f(j) + sum_j (t_j^(-5/2) - 1) F_f(j): the first sum
+// is formed once per tile in FP32, so only the small second one passes through the tensor
+// core, as FP16 pairs (hi + lo, 22 bits) of both factors with FP32 accumulation.  The
+// result of a tile is folded into the running sums as in the pair sweep.
+//
+// Bound and layout.  Per pair: 7 packed FP32 lanes' worth of FMA-pipe work and one rsqrt for
+// the weight, two conversions and a subtraction for its FP16 pair, one word of TMEM written;
+// the products (3 x 29 columns per pair) keep the tensor core a quarter busy.  The loop is
+// bound by issue slots and the FMA pipe (65% and 62% busy).  A thread owns two targets, one
+// row in each of two 128-row accumulators, and takes sources in pairs, so that a packed
+// register pair is one operand word and the source data is not duplicated; four warpgroups
+// per block work at their own pace on a shared ring of source tiles.  A chunk is 32 sources
+// (32 TMEM columns, the accumulators take the other 32 of a tile's 64); the last warp of a
+// group to store its rows issues the chunk's twelve MMAs while the others go on.
+// 400,000 particles onto themselves, compensated: 161 ms by the pair sweep alone, 70 ms so
+// (2.3e12 pairs/s); 100,000: 10.4 and 5.2 ms.
+//
+// A (target group, tile) pair takes this path when the tile's radius is at most FAR_TAU of
+// its centre's distance to the group's boxes and every pair is at least 7 sigma apart (the
+// point-vortex form); all others go to the pair sweep.  far_mask_kernel decides once, and
+// both launches walk the unit lists that it leaves.
+#pragma once
+
+#include "vpm_common.cuh"
+#include "vpm_internal.h"
+
+namespace vpm {
+
+constexpr int FAR_GROUP = 256;                   // targets per far group (a warpgroup, two per thread)
+constexpr int FAR_GROUPS = TGT_TILE / FAR_GROUP; // groups of a target tile
+constexpr unsigned FAR_ALL = (1u << FAR_GROUPS) - 1u;
+// Cost in the pair sweep of a warp's tile within 7 sigma, against one of a tile beyond.
+constexpr int NEAR_COST = 3;
+// Acceptance ratio.  The error does not depend on it where it was measured (0.2 to 0.6: u
+// 1.31e-7 to 1.34e-7, grad u 1.83e-7 throughout on the 100,000-particle hover wake, whose
+// error comes from the near pairs), since every pair is evaluated at any ratio; beyond 0.5
+// the weights (up to 31 there) and the cancellation in t grow and little time is gained
+// (hover wake, 100,000: 7.20 ms at 0.2, 6.23 at 0.33, 5.88 at 0.5, 5.63 at 0.6).
+constexpr float FAR_TAU = 0.5f;
+// (1,024-target, 128-source) units from which the far sweep is used: below, packing and
+// listing (about 40 us) cost more than it saves.  1,280 control points, velocity only:
+// 100,000 sources (1,564 units) 176 us without it and 185 us with it, 150,000 (2,344 units)
+// 240 and 229 us.
+constexpr long long FAR_MIN_UNITS = 2048;
+constexpr long long FAR_MAX_UNITS = 1LL << 26;   // ... and to which (the unit lists take up to 44 bytes each)
+// Particles onto themselves: smallest count put in curve order and swept this way (right-hand
+// side of the BVI wake: 16,000 particles 819 us without and 744 us with it, 12,000 particles
+// 611 and 638 us; hover wake 679 and 690 us, 488 and 572 us).
+constexpr int FAR_SORT_MIN = 16384;
+constexpr int FAR_BND_BLOCKS = 128;              // partial boxes of the curve's bounding cube
+constexpr int FAR_KCH = 2048;                    // source tiles per block of the mask and list kernels
+constexpr float FAR_FSCALE = 256.f;              // features are scaled by this before their FP16 split
+
+// Packed far tile: FP16 features hi then lo in the tensor core's K-major core-matrix
+// order, the scaled offsets in source pairs, the header.
+template <bool GRAD>
+struct FarTile {
+    static constexpr int N = GRAD ? 32 : 16;              // feature columns (29 / 6 used)
+    static constexpr int NF = GRAD ? 29 : 6;
+    static constexpr int FEAT = SRC_TILE * N * 2;         // bytes of one FP16 half
+    static constexpr int OFF_D = 2 * FEAT;                // float4 per source pair: (dx,dx,dy,dy) (dz,dz,q,q)
+    static constexpr int OFF_H = OFF_D + SRC_TILE * 16;   // header: N feature sums, then cx, cy, cz, a, gamma
+    static constexpr int BYTES = OFF_H + 256;
+};
+constexpr size_t far_tile_bytes(bool grad) { return grad ? FarTile<true>::BYTES : FarTile<false>::BYTES; }
+
+// A list of units ordered by target tile: (source tile << 4 | group mask, cost of the
+// units before it); the pair sweep's is ordered by group and holds the source tile alone.  A unit's cost is the number of its groups in the tensor-core list; in
+// the pair sweep's the number of the group's warps, those within 7 sigma counted NEAR_COST times.  The cost line is cut into equal ranges, one per block (at most B of them, and
+// at least a whole unit long, so that every range holds the start of one); block b runs the
+// units whose cost starts in its range and writes one partial sum per target tile into
+// slot b + t.
+struct UnitList {
+    const uint2* list;
+    const int2* off;  // (entries, cost) before each (target tile, chunk); [TT * KY + 1]
+    int TT, KY, B;
+    int max_cost;     // of one unit
+
+    __device__ __forceinline__ int end(int t) const { return off[(t + 1) * KY].x; }
+    __device__ __forceinline__ int blocks(int tot) const { return max(1, min(B, tot / max_cost)); }
+    // Block owning the unit whose cost starts at c.
+    __device__ __forceinline__ int block_of(long long c, int tot) const
+    {
+        return (int)(((c + 1) * blocks(tot) - 1) / tot);
+    }
+    // First index in [0, n) with key(index) >= v (n if none), key nondecreasing, by a whole warp:
+    // 32 probes a round instead of one, since each round waits for memory.
+    template <class Key>
+    static __device__ __forceinline__ int warp_lower_bound(int n, long long v, Key key)
+    {
+        const int lane = threadIdx.x & 31;
+        int a = 0, z = n;  // the answer lies in [a, z]
+        while (a < z) {
+            const int step = (z - a + 31) / 32, q = a + lane * step;
+            const bool below = q < z && (long long)key(q) < v;
+            const int k = __popc(__ballot_sync(0xffffffffu, below));  // probes 0 .. k-1 are below
+            if (k == 0) return a;
+            const int last = a + (k - 1) * step;
+            z = min(z, a + k * step);
+            a = last + 1;
+        }
+        return a;
+    }
+    // The entries [lo, hi) of block b and the target tile of the first; by a whole warp.
+    __device__ __forceinline__ void range(int b, int& lo, int& hi, int& t) const
+    {
+        const int2 tot = off[TT * KY];
+        const int nb = blocks(tot.y);
+        lo = hi = t = 0;
+        if (b >= nb) return;
+        const uint2* l = list;
+        auto cost = [l](int q) { return (int)l[q].y; };
+        lo = warp_lower_bound(tot.x, (long long)b * tot.y / nb, cost);
+        hi = warp_lower_bound(tot.x, (long long)(b + 1) * tot.y / nb, cost);
+        const int2* o = off;
+        const int ky = KY;
+        t = warp_lower_bound(TT, (long long)lo + 1, [o, ky](int q) { return o[(q + 1) * ky].x; });
+    }
+};
+
+struct FarArgs {
+    const float4* tgt;
+    int n_tgt;
+    const unsigned char* tiles;
+    UnitList ul;
+    float* part;
+    int* dev_err;
+};
+
+// Hilbert-curve order of n particles (sorted position -> index, in SweepPlan::off_perm).
+cudaError_t far_sort_bytes(int n, size_t* bytes);
+cudaError_t run_far_sort(const SweepPlan& p, char* ws, const float4* pos, int n, cudaStream_t st);
+cudaError_t run_far_pack(const float4* pos, const float4* str, int n, const float4* box, int SP, bool grad,
+                         unsigned char* tiles, cudaStream_t st);
+cudaError_t run_far_lists(const float4* tgt, int n_tgt, const unsigned char* tiles, int SP, int TT, bool grad,
+                          const float4* pbox, float far2, unsigned* mask, int2* cnt, uint2* near_list, int2* near_off,
+                          uint2* far_list, int2* far_off, cudaStream_t st);
+cudaError_t run_far_sweep(const FarArgs& A, bool grad, bool comp, cudaStream_t st);
+
+}  // namespace vpm

@@ -36,7 +36,7 @@ struct Carve {
 
 int sm_count();
 int* dev_err_ptr();          // device error word of the current device
-int sweep_blocks(bool grad, bool comp, bool stretch, bool segments = false);  // resident sweep blocks (current device)
+int sweep_blocks(bool grad, bool comp, bool stretch, int kind = 0);  // resident sweep blocks (current device)
 int adjoint_blocks(bool comp);
 
 struct SweepPlan {
@@ -48,7 +48,16 @@ struct SweepPlan {
     bool mixed = false;  // particle and segment tiles in one launch (small problems)
     StreamK sk{};        // particle tiles, and the segment tiles when mixed (one launch)
     StreamK sks{};       // otherwise the segment tiles (a launch of their own)
+    // Far units on the tensor cores (vpm_far.cuh); the particle launch then walks the others.
+    bool far = false;
+    int KY = 0, B_near = 0, B_far = 0;  // list chunks per target tile, blocks of the two launches
     size_t off_psrc = 0, off_pbox = 0, off_ssrc = 0, off_sbox = 0, off_part = 0, off_part_s = 0, bytes = 0;
+    // Particles onto themselves: the particles are put in Hilbert-curve order first
+    bool sort = false;
+    size_t off_bnd = 0, off_key = 0, off_key2 = 0, off_idx = 0, off_perm = 0, off_cub = 0, cub_bytes = 0, off_spos = 0,
+           off_sstr = 0, off_obox = 0;
+    size_t off_ftile = 0, off_fmask = 0, off_fcnt = 0, off_nlist = 0, off_noff = 0, off_flist = 0, off_foff = 0,
+           off_part_f = 0, off_part_n = 0;
 };
 
 // Plans a particle + segment sweep onto `n_tgt` targets from a workspace carve: the
@@ -56,7 +65,7 @@ struct SweepPlan {
 // each with its own partial sums, or in one (sk) for a small problem; fills the
 // sub-buffer offsets.
 SweepPlan plan_sweep(int64_t n_tgt, int64_t n_src, int64_t m_seg, bool grad, bool comp, Carve& cv,
-                     bool stretch = false);
+                     bool stretch = false, bool allow_far = true);
 
 // Launches packing, the sweep and the reduction/epilogue.
 struct EpilogueOut {

@@ -23,14 +23,18 @@
 // targets there are.  Far from a warp's 64 targets (the tile's bounding box more
 // than 7 sigma from both of the warp's two target boxes) the blob kernel equals
 // the point-vortex kernel to FP32 precision, so far tiles run the 1/r^3 form with
-// one rsqrt; near tiles evaluate the regularised kernel exactly per pair.  Each tile's sums start from zero and are folded into a
+// one rsqrt; near tiles evaluate the regularised kernel for the sources within 7 sigma of
+// the warp's boxes.  In larger problems the tiles that are far and compact run on the
+// tensor cores instead (vpm_far.cuh), over particles in curve order.  Each tile's sums start from zero and are folded into a
 // per-thread running sum kept in shared memory: a compensated (hi, lo) pair with
 // Knuth's two-sum, or a plain sum, so long source lists keep a tile-sized error.
 #include <math.h>
 
+#include <algorithm>
 #include <mutex>
 
 #include "vpm_common.cuh"
+#include "vpm_far.cuh"
 #include "vpm_internal.h"
 #include "vpm_kernel.cuh"
 
@@ -49,6 +53,22 @@ __device__ __forceinline__ void particle_tile(Acc<GRAD, STRETCH>& a, const float
     } else {
 #pragma unroll 2
         for (int j = 0; j < cnt; ++j) particle_source<GRAD, STRETCH, NEAR>(a, s + j * P_F4, X, Y, Z, nc, o);
+    }
+}
+
+// The sources of a particle tile selected by `keep` (bit j of keep[h]: source 32 h + j).
+template <bool GRAD, bool STRETCH, bool NEAR>
+__device__ __forceinline__ void particle_subset(Acc<GRAD, STRETCH>& a, const float4* __restrict__ s,
+                                                const unsigned (&keep)[SRC_TILE / 32], bool invert, int cnt, f2 X,
+                                                f2 Y, f2 Z, const NearConst& nc, const Own& o)
+{
+#pragma unroll 1
+    for (int h = 0; h < SRC_TILE / 32; ++h) {
+        unsigned m = h == 0 ? keep[0] : h == 1 ? keep[1] : h == 2 ? keep[2] : keep[3];
+        const int left = cnt - 32 * h;
+        if (invert) m = ~m & (left >= 32 ? 0xffffffffu : left > 0 ? (1u << left) - 1u : 0u);
+        for (const float4* sh = s + 32 * h * P_F4; m; m &= m - 1)
+            particle_source<GRAD, STRETCH, NEAR>(a, sh + (__ffs(m) - 1) * P_F4, X, Y, Z, nc, o);
     }
 }
 
@@ -90,17 +110,23 @@ __device__ __forceinline__ void finish_tile(Acc<GRAD, STRETCH>& a, const Acc<GRA
 // ---------------------------------------------------------------------------
 // Packing kernels (one thread per source slot, 128 per block = one tile).
 // ---------------------------------------------------------------------------
+// perm (may be null): the order in which to take the particles, which are then also written
+// out in that order.
 __global__ void __launch_bounds__(SRC_TILE) pack_particles_kernel(const float4* __restrict__ pos,
                                                                   const float4* __restrict__ str, int n,
+                                                                  const int* __restrict__ perm,
+                                                                  float4* __restrict__ spos, float4* __restrict__ sstr,
                                                                   float4* __restrict__ out, float4* __restrict__ box)
 {
     const int j = blockIdx.x * SRC_TILE + threadIdx.x;
     const bool valid = j < n;
     float x = 0.f, y = 0.f, z = 0.f, gx = 0.f, gy = 0.f, gz = 0.f;
     if (valid) {
-        const float4 p = pos[j], g = str[j];
+        const int i = perm ? perm[j] : j;
+        const float4 p = pos[i], g = str[i];
         x = p.x, y = p.y, z = p.z;
         gx = g.x, gy = g.y, gz = g.z;
+        if (perm) spos[j] = p, sstr[j] = g;
     }
     float4* o = out + (size_t)j * P_F4;
     o[0] = make_float4(-x, -x, -y, -y);
@@ -232,12 +258,12 @@ struct SweepArgs {
     int vn;
     int core_pos;  // the segment core is > 0
     StreamK sk;
+    UnitList ul;  // SWEEP_NEAR: the listed units
     NearConst nc;
     float* part;
     int* dev_err;
 };
 
-constexpr int BUF_F4 = SRC_TILE * S_F4 + 2;  // the larger tile format + the tile's bounding box
 constexpr uint64_t WAIT_LIMIT = 2000000000ull;  // 2 s of wall time
 
 template <bool GRAD, bool STRETCH>
@@ -246,103 +272,162 @@ __host__ __device__ constexpr int n_rows()
     return Acc<GRAD, STRETCH>::N;
 }
 
-// Dynamic shared memory: SWEEP_STAGES source tiles, then the running sums of the
-// consumer threads, [row][hi|lo][thread] as float2 (the two targets).
-template <bool GRAD, bool COMP, bool STRETCH>
-__host__ __device__ constexpr size_t sweep_smem_bytes()
-{
-    return (size_t)SWEEP_STAGES * BUF_F4 * 16 + (size_t)n_rows<GRAD, STRETCH>() * (COMP ? 2 : 1) * SWEEP_CW * 32 * 8;
-}
 
 // KIND: the source tiles a launch sweeps.  SWEEP_PARTICLES takes particle tiles and,
 // in the one-launch plan of small problems, segment tiles one segment at a time;
 // SWEEP_SEGMENTS takes only segment tiles, including those packed as closed rings.
 // The ring loop needs more registers than the particle loop; in a launch of its own
-// it costs the particle tiles nothing.  (Measured: the particle launch compiled
+// it costs the particle tiles nothing.  SWEEP_NEAR takes the particle tiles of a unit
+// list: those the tensor-core sweep (vpm_far.cuh) leaves.  They cluster (a source tile is
+// near a few neighbouring target groups), so each warpgroup takes its own range of
+// (256-target group, source tile) units: with blocks of 1,024 targets three quarters of
+// the warps had nothing to do.  (Measured: the particle launch compiled
 // without its segment loop is allocated fewer registers and runs 4% slower.)
-constexpr int SWEEP_PARTICLES = 0, SWEEP_SEGMENTS = 1;
+constexpr int SWEEP_PARTICLES = 0, SWEEP_SEGMENTS = 1, SWEEP_NEAR = 2;
+constexpr int SWEEP_KINDS = 3;
+
+// A ring of source stages serves a team of warps: the whole block, or with SWEEP_NEAR
+// each warpgroup its own.
+template <int KIND>
+struct Ring {
+    static constexpr bool LIST = KIND == SWEEP_NEAR;
+    static constexpr int TEAMS = LIST ? SWEEP_CW / 4 : 1, WARPS = SWEEP_CW / TEAMS;
+    static constexpr int STAGES = LIST ? 2 : SWEEP_STAGES;         // per team
+    static constexpr int BOX = SRC_TILE * (LIST ? P_F4 : S_F4);    // the tile's bounding box, float4s into a stage
+    static constexpr int F4 = BOX + 2;
+    static constexpr int TGT = LIST ? FAR_GROUP : TGT_TILE;        // targets of a team
+};
+
+// Dynamic shared memory: the source stages, then the running sums of the consumer
+// threads, [row][hi|lo][thread] as float2 (the two targets).
+template <bool GRAD, bool COMP, bool STRETCH, int KIND>
+__host__ __device__ constexpr size_t sweep_smem_bytes()
+{
+    return (size_t)Ring<KIND>::TEAMS * Ring<KIND>::STAGES * Ring<KIND>::F4 * 16 +
+           (size_t)n_rows<GRAD, STRETCH>() * (COMP ? 2 : 1) * SWEEP_CW * 32 * 8;
+}
 
 template <bool GRAD, bool COMP, bool STRETCH, int KIND>
 __global__ void __launch_bounds__(SWEEP_TPB, 1) sweep_kernel(const SweepArgs A)
 {
+    using R = Ring<KIND>;
+    constexpr bool LIST = R::LIST;
+    constexpr int NST = R::TEAMS * R::STAGES;
     extern __shared__ __align__(128) float4 dsm[];
-    __shared__ __align__(8) uint64_t full[SWEEP_STAGES];
-    __shared__ int released[SWEEP_STAGES];
-    __shared__ int issued_round[SWEEP_STAGES];  // round of the latest copy into each stage
+    __shared__ __align__(8) uint64_t full[NST];
+    __shared__ int released[NST];
+    __shared__ int issued_round[NST];  // round of the latest copy into each stage
     __shared__ float wbox[SWEEP_CW][12];
     constexpr int NR = n_rows<GRAD, STRETCH>();
     constexpr int NT = SWEEP_CW * 32;
-    float4* stage = dsm;
-    f2* run = reinterpret_cast<f2*>(dsm + SWEEP_STAGES * BUF_F4);  // [NR][COMP?2:1][NT]
-
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int team = warp / R::WARPS, s0 = team * R::STAGES;  // this team's first stage
+    float4* stage = dsm;
+    f2* run = reinterpret_cast<f2*>(dsm + NST * R::F4);  // [NR][COMP?2:1][NT]
+
     const StreamK& sk = A.sk;
-    const int b = blockIdx.x;
-    const long long lo_b = sk.lo(b), hi_b = sk.lo(b + 1);
+    const UnitList& ul = A.ul;
+    const int b = blockIdx.x * R::TEAMS + team;
+    long long lo_b, hi_b;  // this team's range: of the cost line, or of the list's entries
     int t0, k0;
-    sk.first_at_or_after(lo_b, t0, k0);
-    if (t0 >= sk.TT || sk.unit_start(t0, k0) >= hi_b) return;  // block owns no unit (uniform)
+    if constexpr (LIST) {
+        __shared__ int range_s[R::TEAMS][3];
+        if (warp % R::WARPS == 0) {
+            int l, h, t;
+            ul.range(b, l, h, t);
+            if (lane == 0) range_s[team][0] = l, range_s[team][1] = h, range_s[team][2] = t;
+        }
+        __syncthreads();
+        lo_b = range_s[team][0], hi_b = range_s[team][1], t0 = range_s[team][2];
+        k0 = 0;
+    } else {
+        lo_b = sk.lo(b), hi_b = sk.lo(b + 1);
+        sk.first_at_or_after(lo_b, t0, k0);
+        if (t0 >= sk.TT || sk.unit_start(t0, k0) >= hi_b) return;  // block owns no unit (uniform)
+    }
     const int nunits = sk.np + sk.ns;
 
     // Copies source unit kk (and its bounding box) into stage s, completing on full[s].
     auto issue = [&](int kk, int s, int round) {
         issued_round[s] = round;
         fence_proxy_async_smem();
-        if (kk < sk.np) {
+        if (LIST || kk < sk.np) {
             const uint32_t bytes = SRC_TILE * P_F4 * 16;
             mbar_expect_tx(&full[s], bytes + 32);
-            bulk_g2s(stage + (size_t)s * BUF_F4, A.psrc + (size_t)kk * SRC_TILE * P_F4, bytes, &full[s]);
-            bulk_g2s(stage + (size_t)s * BUF_F4 + SRC_TILE * S_F4, A.pbox + 2 * kk, 32, &full[s]);
+            bulk_g2s(stage + (size_t)s * R::F4, A.psrc + (size_t)kk * SRC_TILE * P_F4, bytes, &full[s]);
+            bulk_g2s(stage + (size_t)s * R::F4 + R::BOX, A.pbox + 2 * kk, 32, &full[s]);
         } else {
             const uint32_t bytes = SRC_TILE * S_F4 * 16;
             mbar_expect_tx(&full[s], bytes + 32);
-            bulk_g2s(stage + (size_t)s * BUF_F4, A.ssrc + (size_t)(kk - sk.np) * SRC_TILE * S_F4, bytes, &full[s]);
-            bulk_g2s(stage + (size_t)s * BUF_F4 + SRC_TILE * S_F4, A.sbox + 2 * (kk - sk.np), 32, &full[s]);
+            bulk_g2s(stage + (size_t)s * R::F4, A.ssrc + (size_t)(kk - sk.np) * SRC_TILE * S_F4, bytes, &full[s]);
+            bulk_g2s(stage + (size_t)s * R::F4 + R::BOX, A.sbox + 2 * (kk - sk.np), 32, &full[s]);
         }
     };
-    // The unit `ahead` places after (t, k) in this block's run, if the block owns it.
-    auto unit_ahead = [&](int t, int k, int ahead, int& kk) {
+    // The unit `ahead` places after the i-th, (t, k), in this team's run, if the team owns it.
+    auto unit_ahead = [&](int i, int t, int k, int ahead, int& kk) {
+        if constexpr (LIST) {
+            const long long q = lo_b + i + ahead;
+            if (q >= hi_b) return false;
+            kk = (int)ul.list[q].x;
+            return true;
+        }
         for (int q = 0; q < ahead; ++q)
             if (++k == nunits) k = 0, ++t;
         kk = k;
         return t < sk.TT && sk.unit_start(t, k) < hi_b;
     };
 
-    if (tid == 0) {
-        for (int s = 0; s < SWEEP_STAGES; ++s) {
-            mbar_init(&full[s], 1);
-            released[s] = 0;
+    if (warp % R::WARPS == 0 && lane == 0) {
+        for (int s = 0; s < R::STAGES; ++s) {
+            mbar_init(&full[s0 + s], 1);
+            released[s0 + s] = 0;
+            issued_round[s0 + s] = -1;
         }
         mbar_fence_init();
-        for (int s = 0; s < SWEEP_STAGES; ++s) {  // first fill of the ring
+        for (int s = 0; s < R::STAGES; ++s) {  // first fill of the ring
             int kk;
-            if (!unit_ahead(t0, k0, s, kk)) break;
-            issue(kk, s, 0);
+            if (!unit_ahead(0, t0, k0, s, kk)) break;
+            issue(kk, s0 + s, 0);
         }
     }
     __syncthreads();
+    if (LIST && lo_b >= hi_b) return;  // team owns no unit
 
     // ---------------- consumers ----------------
     const int ct = warp * 32 + lane;  // consumer thread index
     Acc<GRAD, STRETCH> acc;
     f2 X = zero2(), Y = zero2(), Z = zero2();
     int t = t0, k = k0, cur_t = -1;
+    int t_end = 0;  // LIST: end of target group t's entries
+    if constexpr (LIST) {
+        t_end = ul.end(t);
+        k = (int)ul.list[lo_b].x;
+    }
     auto zero_run = [&]() {
 #pragma unroll
         for (int q = 0; q < NR * (COMP ? 2 : 1); ++q) run[q * NT + ct] = zero2();
     };
     zero_run();
     for (int i = 0;; ++i) {
-        const int s = i % SWEEP_STAGES, r = i / SWEEP_STAGES;
+        const int s = s0 + i % R::STAGES, r = i / R::STAGES;
         int nt = t, nk = k + 1;
-        if (nk == nunits) {
-            nk = 0;
-            ++nt;
+        bool has_next;
+        if constexpr (LIST) {
+            has_next = lo_b + i + 1 < hi_b;
+            if (has_next) {
+                nk = (int)ul.list[lo_b + i + 1].x;
+                while (lo_b + i + 1 >= t_end) t_end = ul.end(++nt);
+            }
+        } else {
+            if (nk == nunits) {
+                nk = 0;
+                ++nt;
+            }
+            has_next = nt < sk.TT && sk.unit_start(nt, nk) < hi_b;
         }
-        const bool has_next = nt < sk.TT && sk.unit_start(nt, nk) < hi_b;
         if (t != cur_t) {  // new target tile: this warp's 64 targets, their box and strengths
             cur_t = t;
-            const int i0 = t * TGT_TILE + warp * 64 + lane, i1 = i0 + 32;
+            const int i0 = t * R::TGT + (warp % R::WARPS) * 64 + lane, i1 = i0 + 32;
             float4 p0 = make_float4(0.f, 0.f, 0.f, 0.f), p1 = p0;
             const bool v0 = i0 < A.n_tgt, v1 = i1 < A.n_tgt;
             if (v0) p0 = A.tgt[i0];
@@ -353,23 +438,23 @@ __global__ void __launch_bounds__(SWEEP_TPB, 1) sweep_kernel(const SweepArgs A)
             warp_two_boxes(make_float3(p0.x, p0.y, p0.z), v0, make_float3(p1.x, p1.y, p1.z), v1, wbox[warp]);
         }
         if (!mbar_wait_bounded(&full[s], r & 1, A.dev_err, WAIT_LIMIT)) {
-            // latched; the results are invalid.  Let this block's copies in flight land
+            // latched; the results are invalid.  Let this team's copies in flight land
             // (bounded) before its shared memory is released, then leave.
             if (lane == 0)
-                for (int q = 0; q < SWEEP_STAGES; ++q)
-                    mbar_wait_bounded(&full[q], issued_round[q] & 1, A.dev_err, WAIT_LIMIT);
+                for (int q = s0; q < s0 + R::STAGES; ++q)
+                    if (issued_round[q] >= 0) mbar_wait_bounded(&full[q], issued_round[q] & 1, A.dev_err, WAIT_LIMIT);
             break;
         }
 
-        const float4* src = stage + (size_t)s * BUF_F4;
+        const float4* src = stage + (size_t)s * R::F4;
         // Far particle tiles and segment tiles accumulate without the stretching rows and
         // the target strengths (fewer live registers in their loops); finish_tile adds the
         // stretching from the tile's sums afterwards.  Near particle tiles accumulate the
         // stretching pair by pair (it cancels there) with the strengths loaded for them.
-        const int ti0 = t * TGT_TILE + warp * 64 + lane, ti1 = ti0 + 32;
-        if (KIND == SWEEP_PARTICLES && k < sk.np) {
+        const int ti0 = t * R::TGT + (warp % R::WARPS) * 64 + lane, ti1 = ti0 + 32;
+        if (LIST || (KIND == SWEEP_PARTICLES && k < sk.np)) {
             const int cnt = min(SRC_TILE, A.n_src - k * SRC_TILE);
-            const float4 tlo = src[SRC_TILE * S_F4], thi = src[SRC_TILE * S_F4 + 1];
+            const float4 tlo = src[R::BOX], thi = src[R::BOX + 1];
             if (boxes_near(wbox[warp], tlo, thi, A.nc.far2)) {
                 Own own{zero2(), zero2(), zero2()};
                 if (STRETCH) {
@@ -380,8 +465,23 @@ __global__ void __launch_bounds__(SWEEP_TPB, 1) sweep_kernel(const SweepArgs A)
                     own.gy = make_float2(g0.y, g1.y);
                     own.gz = make_float2(g0.z, g1.z);
                 }
-                acc.zero();
-                particle_tile<GRAD, STRETCH, true>(acc, src, cnt, X, Y, Z, A.nc, own);
+                // Sources at least 7 sigma from both of the warp's boxes take the point-vortex
+                // form (and give their stretching from their sums, as a far tile does)
+                unsigned keep[SRC_TILE / 32];
+#pragma unroll
+                for (int h = 0; h < SRC_TILE / 32; ++h) {
+                    const int j = 32 * h + lane;
+                    const float4 q0 = src[j * P_F4], q1 = src[j * P_F4 + 1];
+                    const float4 pt = make_float4(-q0.x, -q0.z, -q1.x, 0.f);
+                    keep[h] = __ballot_sync(0xffffffffu, j < cnt && boxes_near(wbox[warp], pt, pt, A.nc.far2 * 1.00001f));
+                }
+                {
+                    Acc<GRAD, false> tf;
+                    tf.zero();
+                    particle_subset<GRAD, false, false>(tf, src, keep, true, cnt, X, Y, Z, A.nc, Own{});
+                    finish_tile<GRAD, STRETCH>(acc, tf, A.tstr, ti0, ti1, A.n_tgt);
+                }
+                particle_subset<GRAD, STRETCH, true>(acc, src, keep, false, cnt, X, Y, Z, A.nc, own);
             } else {
                 Acc<GRAD, false> tf;
                 tf.zero();
@@ -390,7 +490,7 @@ __global__ void __launch_bounds__(SWEEP_TPB, 1) sweep_kernel(const SweepArgs A)
             }
         } else {
             const int cnt = min(SRC_TILE, A.m_seg - (k - sk.np) * SRC_TILE);
-            const float4 tlo = src[SRC_TILE * S_F4], thi = src[SRC_TILE * S_F4 + 1];
+            const float4 tlo = src[R::BOX], thi = src[R::BOX + 1];
             const float margin = 1e-3f * tlo.w;
             const bool safe = A.core_pos && margin > 0.f && !boxes_near(wbox[warp], tlo, thi, margin * margin);
             Acc<GRAD, false> tf;
@@ -408,13 +508,13 @@ __global__ void __launch_bounds__(SWEEP_TPB, 1) sweep_kernel(const SweepArgs A)
             finish_tile<GRAD, STRETCH>(acc, tf, A.tstr, ti0, ti1, A.n_tgt);
         }
         __syncwarp();
-        if (lane == 0) {  // the last warp to finish with stage s refills it with unit i + SWEEP_STAGES
+        if (lane == 0) {  // the last warp to finish with stage s refills it with unit i + STAGES
             __threadfence_block();
-            if (atomicAdd(&released[s], 1) == SWEEP_CW - 1) {
+            if (atomicAdd(&released[s], 1) == R::WARPS - 1) {
                 released[s] = 0;
                 __threadfence_block();
                 int kk;
-                if (unit_ahead(t, k, SWEEP_STAGES, kk)) issue(kk, s, r + 1);
+                if (unit_ahead(i, t, k, R::STAGES, kk)) issue(kk, s, r + 1);
             }
         }
         // fold this tile's sums into the running sums
@@ -429,15 +529,15 @@ __global__ void __launch_bounds__(SWEEP_TPB, 1) sweep_kernel(const SweepArgs A)
                 run[q * NT + ct] = add2(run[q * NT + ct], acc.v[q]);
             }
         }
-        if (!has_next || nt != t) {  // this warp's partial of target tile t
-            float* P = A.part + ((size_t)(b + t) * (COMP ? 2 * NR : NR)) * TGT_TILE + warp * 64 + lane;
+        if (!has_next || nt != t) {  // this warp's partial of target tile (LIST: group) t
+            float* P = A.part + ((size_t)(b + t) * (COMP ? 2 * NR : NR)) * R::TGT + (warp % R::WARPS) * 64 + lane;
 #pragma unroll
             for (int q = 0; q < NR * (COMP ? 2 : 1); ++q) {
                 const f2 v = run[q * NT + ct];
                 // rows: hi of every accumulator first, then lo
                 const int row = COMP ? ((q & 1) ? NR + (q >> 1) : (q >> 1)) : q;
-                P[(size_t)row * TGT_TILE] = v.x;
-                P[(size_t)row * TGT_TILE + 32] = v.y;
+                P[(size_t)row * R::TGT] = v.x;
+                P[(size_t)row * R::TGT + 32] = v.y;
             }
             zero_run();
         }
@@ -448,14 +548,19 @@ __global__ void __launch_bounds__(SWEEP_TPB, 1) sweep_kernel(const SweepArgs A)
 }
 
 // ---------------------------------------------------------------------------
-// Reduction of the stream-K partial sums (fixed order, FP64) and epilogue.
+// Reduction of the stream-K partial sums (fixed order) and epilogue.
 // ---------------------------------------------------------------------------
 struct EpiArgs {
     StreamK sk, sks;  // the particle and the segment launch
     const float* part;
     const float* part_s;
+    int far;            // the particle units are split between two lists
+    UnitList uln, ulf;  // ... those of the particle launch and of the tensor-core launch
+    const float* part_f;
+    int ncomp_f;        // rows of the tensor-core launch (no stretching rows)
     int n, ncomp, comp;
     EpilogueOut o;
+    const int* perm;  // where target i's outputs go (null: i)
     int* dev_err;
 };
 
@@ -464,11 +569,18 @@ __device__ __forceinline__ void check_finite(int* dev_err, double v)
     if (!isfinite(v)) atomicOr(dev_err, DEV_ERR_NONFINITE);
 }
 
+// PARTS threads of a block share a target's partial sums (a few targets have many, one
+// per block of a sweep), each folding every PARTS-th; 256 / PARTS targets per block.
+// Latency bound: a target's partial sums are read one after the other (1,280 control
+// points, 152 partial sums each: 231 us with one thread per target, 31 us with eight).
+template <int PARTS>
 __global__ void __launch_bounds__(256) epilogue_kernel(const EpiArgs E)
 {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= E.n) return;
-    const int t = i / TGT_TILE, l = i % TGT_TILE;
+    constexpr int TB = 256 / PARTS;
+    const int part_i = threadIdx.x / TB;
+    const int i = blockIdx.x * TB + threadIdx.x % TB;
+    if (PARTS == 1 && i >= E.n) return;
+    const int t = min(i, E.n - 1) / TGT_TILE, l = i % TGT_TILE;
     // The partial sums are folded in FP32 double-float arithmetic (hi by Knuth's
     // two-sum, the low words added apart: about 48 bits) and converted to FP64 once
     // per row; the FP64 pipe, a small fraction of the FP32 rate here, keeps only the
@@ -476,8 +588,46 @@ __global__ void __launch_bounds__(256) epilogue_kernel(const EpiArgs E)
     float H[17], Lw[17];
 #pragma unroll
     for (int c = 0; c < 17; ++c) H[c] = 0.f, Lw[c] = 0.f;
+    auto add = [&](const float* P, int ncomp, int ld) {
+#pragma unroll
+        for (int c = 0; c < 17; ++c) {  // a constant bound keeps the sums in registers
+            if (c < ncomp) {
+                float sum, err;
+                two_sum(H[c], P[(size_t)c * ld], sum, err);
+                H[c] = sum;
+                Lw[c] = __fadd_rn(Lw[c], err);
+                if (E.comp) Lw[c] = __fadd_rn(Lw[c], P[(size_t)(ncomp + c) * ld]);
+            }
+        }
+    };
+    auto add_list = [&](const UnitList& ul, const float* part, int ncomp, int ld) {  // ld targets per list row
+        const int t = min(i, E.n - 1) / ld, l = i % ld;
+        const int2 s = ul.off[t * ul.KY], e = ul.off[(t + 1) * ul.KY];
+        if (s.x >= e.x) return;
+        const int tot = ul.off[ul.TT * ul.KY].y;
+        const int b0 = ul.block_of(s.y, tot), b1 = ul.block_of(ul.list[e.x - 1].y, tot), rows = E.comp ? 2 * ncomp : ncomp;
+        for (int b = b0 + part_i; b <= b1; b += PARTS) add(part + (size_t)(b + t) * rows * ld + l, ncomp, ld);
+    };
+    if (E.far) {
+        add_list(E.ulf, E.part_f, E.ncomp_f, TGT_TILE);
+        if (E.ncomp == 17) {
+            // the far units' transposed stretching (times 4 pi) from their sums, Gamma_i x S - 3 G'^T Gamma_i
+            const float4 g = reinterpret_cast<const float4*>(E.o.str)[min(i, E.n - 1)];
+            double v[14];
+#pragma unroll
+            for (int c = 3; c < 14; ++c) v[c] = (double)H[c] + (double)Lw[c];
+            const double gzz = -(v[6] + v[10]);
+            const double s[3] = {
+                (g.y * v[5] - g.z * v[4]) - 3.0 * (v[6] * g.x + v[9] * g.y + v[12] * g.z),
+                (g.z * v[3] - g.x * v[5]) - 3.0 * (v[7] * g.x + v[10] * g.y + v[13] * g.z),
+                (g.x * v[4] - g.y * v[3]) - 3.0 * (v[8] * g.x + v[11] * g.y + gzz * g.z)};
+#pragma unroll
+            for (int c = 0; c < 3; ++c) H[14 + c] = (float)s[c], Lw[14 + c] = (float)(s[c] - (double)H[14 + c]);
+        }
+        add_list(E.uln, E.part, E.ncomp, FAR_GROUP);
+    }
     // the partial sums of the particle launch, then those of the segment launch
-    for (int launch = 0; launch < 2; ++launch) {
+    for (int launch = E.far ? 1 : 0; launch < 2; ++launch) {
         const StreamK& sk = launch ? E.sks : E.sk;
         const float* part = launch ? E.part_s : E.part;
         const int nunits = sk.np + sk.ns;
@@ -485,24 +635,31 @@ __global__ void __launch_bounds__(256) epilogue_kernel(const EpiArgs E)
         const int b0 = sk.block_of(sk.unit_start(t, 0));
         const int b1 = sk.block_of(sk.unit_start(t, nunits - 1));
         const int rows = E.comp ? 2 * E.ncomp : E.ncomp;
-        for (int b = b0; b <= b1; ++b) {
+        for (int b = b0 + part_i; b <= b1; b += PARTS) {
             const long long lo_b = sk.lo(b), hi_b = sk.lo(b + 1);
             long long c0 = lo_b > (long long)t * sk.C ? lo_b : (long long)t * sk.C;
             int tt, kk;
             sk.first_at_or_after(c0, tt, kk);
             if (tt != t || sk.unit_start(tt, kk) >= hi_b) continue;  // block b ran no unit of tile t
-            const float* P = part + (size_t)(b + t) * rows * TGT_TILE + l;
+            add(part + (size_t)(b + t) * rows * TGT_TILE + l, E.ncomp, TGT_TILE);
+        }
+    }
+    if constexpr (PARTS > 1) {  // fold the parts, in order
+        __shared__ float sh[17][2][256];
 #pragma unroll
-            for (int c = 0; c < 17; ++c) {  // a constant bound keeps the sums in registers
+        for (int c = 0; c < 17; ++c)
+            if (c < E.ncomp) sh[c][0][threadIdx.x] = H[c], sh[c][1][threadIdx.x] = Lw[c];
+        __syncthreads();
+        if (part_i > 0 || i >= E.n) return;
+        for (int p = 1; p < PARTS; ++p)
+#pragma unroll
+            for (int c = 0; c < 17; ++c)
                 if (c < E.ncomp) {
                     float sum, err;
-                    two_sum(H[c], P[(size_t)c * TGT_TILE], sum, err);
+                    two_sum(H[c], sh[c][0][threadIdx.x + p * TB], sum, err);
                     H[c] = sum;
-                    Lw[c] = __fadd_rn(Lw[c], err);
-                    if (E.comp) Lw[c] = __fadd_rn(Lw[c], P[(size_t)(E.ncomp + c) * TGT_TILE]);
+                    Lw[c] = __fadd_rn(__fadd_rn(Lw[c], err), sh[c][1][threadIdx.x + p * TB]);
                 }
-            }
-        }
     }
     double acc[17];
 #pragma unroll
@@ -525,12 +682,13 @@ __global__ void __launch_bounds__(256) epilogue_kernel(const EpiArgs E)
         J[7] = (Sx - 3.0 * acc[13]) * f4pi;
         J[8] = (-3.0 * Gzz) * f4pi;
     }
+    const int d = E.perm ? E.perm[i] : i;
     if (o.mode == 0) {
-        o.u[i] = (float)u0;
-        o.u[E.n + i] = (float)u1;
-        o.u[2 * E.n + i] = (float)u2;
+        o.u[d] = (float)u0;
+        o.u[E.n + d] = (float)u1;
+        o.u[2 * E.n + d] = (float)u2;
         if (o.grad_u)
-            for (int c = 0; c < 9; ++c) o.grad_u[(size_t)c * E.n + i] = (float)J[c];
+            for (int c = 0; c < 9; ++c) o.grad_u[(size_t)c * E.n + d] = (float)J[c];
         if (o.check_finite) {
             check_finite(E.dev_err, u0 + u1 + u2);
             if (o.grad_u) check_finite(E.dev_err, J[0] + J[1] + J[2] + J[3] + J[4] + J[5] + J[6] + J[7] + J[8]);
@@ -561,13 +719,14 @@ __global__ void __launch_bounds__(256) epilogue_kernel(const EpiArgs E)
             s[a] = v;
         }
     }
-    o.dxdt[i] = (float)(u0 + o.uinf[0]);
-    o.dxdt[E.n + i] = (float)(u1 + o.uinf[1]);
-    o.dxdt[2 * E.n + i] = (float)(u2 + o.uinf[2]);
-    o.dGdt[i] = (float)s[0];
-    o.dGdt[E.n + i] = (float)s[1];
-    o.dGdt[2 * E.n + i] = (float)s[2];
-    o.nu_t[i] = (float)nut;
+    o.dxdt[d] = (float)(u0 + o.uinf[0]);
+    o.dxdt[E.n + d] = (float)(u1 + o.uinf[1]);
+    o.dxdt[2 * E.n + d] = (float)(u2 + o.uinf[2]);
+    o.dGdt[d] = (float)s[0];
+    o.dGdt[E.n + d] = (float)s[1];
+    o.dGdt[2 * E.n + d] = (float)s[2];
+    o.nu_t[d] = (float)nut;
+
     if (o.check_finite) check_finite(E.dev_err, u0 + u1 + u2 + s[0] + s[1] + s[2] + nut);
 }
 
@@ -575,12 +734,13 @@ __global__ void __launch_bounds__(256) epilogue_kernel(const EpiArgs E)
 // Particle strength exchange (Eq. 5's diffusion term):
 //   p_i = (2/sigma^2) sum_j nu_ij (v_i Gamma_j - v_j Gamma_i) zeta_sigma(r_ij),
 //   nu_ij = nu + (nu_t,i + nu_t,j)/2, zeta of Eq. 3.
-// Each warp owns 64 consecutive particles (two per lane) with two bounding boxes
-// (split at the largest index-order jump).  It walks the source tiles 32 at a
-// time, one box test per lane, and for every tile within 7 sigma of either box
-// stages the tile (positions, strengths, nu_t) in its own slice of shared memory
-// with coalesced loads, then every lane sums over it.  No block-wide barrier:
-// warps proceed independently.  v_i Gamma_j - v_j Gamma_i is formed from two
+// Each block owns 64 consecutive particles (two per lane of every warp) with two bounding
+// boxes (split at the largest index-order jump).  Its warps walk the source tiles 32 at a
+// time, one box test per lane, and share the tiles within 7 sigma of either box among
+// them, tile by tile: a warp stages its tile (positions, strengths, nu_t) in its own slice
+// of shared memory with coalesced loads, then every lane sums over it; the warps' sums are
+// added in a fixed order.  (One warp per 64 particles left most SMs idle below 50,000
+// particles: 71 us for 2,000 and 86 us for 20,000, 30 and 33 us so.)  v_i Gamma_j - v_j Gamma_i is formed from two
 // rounded products so that the i == j term is exactly zero; pairs beyond 7 sigma
 // get exp(-r^2/2s^2) < 3e-11 and are skipped.
 // ---------------------------------------------------------------------------
@@ -610,9 +770,7 @@ __global__ void __launch_bounds__(PSE_T) pse_kernel(const float4* __restrict__ p
     __shared__ float snt[PSE_W][SRC_TILE];
     __shared__ float wbox[PSE_W][12];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int base_i = (blockIdx.x * PSE_W + warp) * 64;
-    if (base_i >= n) return;  // whole warp past the end
-    const int i0 = base_i + lane, i1 = i0 + 32;
+    const int i0 = blockIdx.x * 64 + lane, i1 = i0 + 32;
     const bool v0 = i0 < n, v1 = i1 < n;
     float4 p0 = make_float4(0.f, 0.f, 0.f, 0.f), p1 = p0, g0 = p0, g1 = p0;
     float nt0 = 0.f, nt1 = 0.f;
@@ -621,13 +779,14 @@ __global__ void __launch_bounds__(PSE_T) pse_kernel(const float4* __restrict__ p
     warp_two_boxes(make_float3(p0.x, p0.y, p0.z), v0, make_float3(p1.x, p1.y, p1.z), v1, wbox[warp]);
     const float base0 = nu + 0.5f * nt0, base1 = nu + 0.5f * nt1;
     float a0x = 0.f, a0y = 0.f, a0z = 0.f, a1x = 0.f, a1y = 0.f, a1z = 0.f;
+    int met = 0;  // tiles in reach so far: warp w takes those with number = w (mod PSE_W)
     for (int tb = 0; tb < ntiles; tb += 32) {
         const int tt = tb + lane;
         const bool near = tt < ntiles && boxes_near(wbox[warp], box[2 * tt], box[2 * tt + 1], cut2);
         unsigned mask = __ballot_sync(0xffffffffu, near);
-        while (mask) {
+        for (; mask; mask &= mask - 1, ++met) {
+            if ((met & (PSE_W - 1)) != warp) continue;
             const int tile = tb + __ffs(mask) - 1;
-            mask &= mask - 1;
             const int j0 = tile * SRC_TILE, cnt = min(SRC_TILE, n - j0);
             // stage the tile; a source at least 7 sigma from both of the warp's target boxes
             // reaches none of its targets and is left out (warp-uniformly, by ballot)
@@ -659,15 +818,47 @@ __global__ void __launch_bounds__(PSE_T) pse_kernel(const float4* __restrict__ p
             }
         }
     }
-    if (v0) {
-        dGdt[i0] += pref * a0x;
-        dGdt[n + i0] += pref * a0y;
-        dGdt[2 * n + i0] += pref * a0z;
+    // the warps' sums in a fixed order, one thread per target
+    __syncthreads();
+    float4* sums = &sp[0][0];  // [PSE_W][64]
+    sums[warp * 64 + lane] = make_float4(a0x, a0y, a0z, 0.f);
+    sums[warp * 64 + 32 + lane] = make_float4(a1x, a1y, a1z, 0.f);
+    __syncthreads();
+    const int i = blockIdx.x * 64 + threadIdx.x;
+    if (threadIdx.x < 64 && i < n) {
+        float4 v = sums[threadIdx.x];
+        for (int w = 1; w < PSE_W; ++w) {
+            const float4 x = sums[w * 64 + threadIdx.x];
+            v.x += x.x, v.y += x.y, v.z += x.z;
+        }
+        dGdt[i] += pref * v.x;
+        dGdt[n + i] += pref * v.y;
+        dGdt[2 * n + i] += pref * v.z;
     }
-    if (v1) {
-        dGdt[i1] += pref * a1x;
-        dGdt[n + i1] += pref * a1y;
-        dGdt[2 * n + i1] += pref * a1z;
+}
+
+// Bounding boxes of the particle tiles in the caller's order.
+__global__ void __launch_bounds__(SRC_TILE) tile_box_kernel(const float4* __restrict__ pos, int n,
+                                                            float4* __restrict__ box)
+{
+    const int j = blockIdx.x * SRC_TILE + threadIdx.x;
+    float v[6] = {INFINITY, INFINITY, INFINITY, INFINITY, INFINITY, INFINITY};  // least of x and of -x
+    if (j < n) {
+        const float4 p = pos[j];
+        v[0] = p.x, v[1] = p.y, v[2] = p.z, v[3] = -p.x, v[4] = -p.y, v[5] = -p.z;
+    }
+    __shared__ float sb[SRC_TILE / 32][6];
+#pragma unroll
+    for (int c = 0; c < 6; ++c) {
+        for (int o = 16; o > 0; o >>= 1) v[c] = fminf(v[c], __shfl_xor_sync(0xffffffffu, v[c], o));
+        if ((threadIdx.x & 31) == 0) sb[threadIdx.x >> 5][c] = v[c];
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int w = 1; w < SRC_TILE / 32; ++w)
+            for (int c = 0; c < 6; ++c) v[c] = fminf(v[c], sb[w][c]);
+        box[2 * blockIdx.x] = make_float4(v[0], v[1], v[2], 0.f);
+        box[2 * blockIdx.x + 1] = make_float4(-v[3], -v[4], -v[5], 0.f);
     }
 }
 
@@ -679,8 +870,8 @@ __device__ int g_dev_err;  // device error word (one instance per device)
 namespace {
 std::mutex g_mu;
 int g_sm[64];
-int g_blocks[64][16];
-bool g_attr[64][16];
+int g_blocks[64][8 * SWEEP_KINDS];
+bool g_attr[64][8 * SWEEP_KINDS];
 }  // namespace
 
 static int cur_dev()
@@ -719,7 +910,7 @@ template <bool G, bool C, bool S, int K>
 static int prepare_kernel(int d)
 {
     const int v = variant(G, C, S, K);
-    const size_t smem = sweep_smem_bytes<G, C, S>();
+    const size_t smem = sweep_smem_bytes<G, C, S, K>();
     {
         std::lock_guard<std::mutex> lk(g_mu);
         if (d >= 0 && d < 64 && g_attr[d][v]) return g_blocks[d][v];
@@ -746,18 +937,21 @@ static int blocks_per_sm_kind(bool g, bool c, bool s)
     return c ? prepare_kernel<false, true, false, K>(d) : prepare_kernel<false, false, false, K>(d);
 }
 
-static int blocks_per_sm(bool g, bool c, bool s, bool segments)
+static int blocks_per_sm(bool g, bool c, bool s, int kind)
 {
-    return segments ? blocks_per_sm_kind<SWEEP_SEGMENTS>(g, c, s) : blocks_per_sm_kind<SWEEP_PARTICLES>(g, c, s);
+    return kind == SWEEP_SEGMENTS ? blocks_per_sm_kind<SWEEP_SEGMENTS>(g, c, s)
+           : kind == SWEEP_NEAR   ? blocks_per_sm_kind<SWEEP_NEAR>(g, c, s)
+                                  : blocks_per_sm_kind<SWEEP_PARTICLES>(g, c, s);
 }
 
-int sweep_blocks(bool grad, bool comp, bool stretch, bool segments)
+int sweep_blocks(bool grad, bool comp, bool stretch, int kind)
 {
     const int sms = sm_count();
-    return blocks_per_sm(grad, comp, stretch && grad, segments) * (sms > 0 ? sms : 1);
+    return blocks_per_sm(grad, comp, stretch && grad, kind) * (sms > 0 ? sms : 1);
 }
 
-SweepPlan plan_sweep(int64_t n_tgt, int64_t n_src, int64_t m_seg, bool grad, bool comp, Carve& cv, bool stretch)
+SweepPlan plan_sweep(int64_t n_tgt, int64_t n_src, int64_t m_seg, bool grad, bool comp, Carve& cv, bool stretch,
+                     bool allow_far)
 {
     SweepPlan p;
     p.n_tgt = (int)n_tgt;
@@ -780,7 +974,7 @@ SweepPlan plan_sweep(int64_t n_tgt, int64_t n_src, int64_t m_seg, bool grad, boo
         sk.C = (long long)sk.np * sk.wp + (long long)sk.ns * sk.ws;
         sk.tot = (long long)sk.TT * sk.C;
         const long long units = (long long)sk.TT * (sk.np + sk.ns);
-        long long B = sweep_blocks(grad, comp, p.stretch, ns > 0);
+        long long B = sweep_blocks(grad, comp, p.stretch, ns > 0 ? SWEEP_SEGMENTS : SWEEP_PARTICLES);
         if (B > units) B = units;
         if (B < 1) B = 1;
         sk.B = (int)B;
@@ -789,7 +983,7 @@ SweepPlan plan_sweep(int64_t n_tgt, int64_t n_src, int64_t m_seg, bool grad, boo
     // kinds of tile in one launch; a larger one gives the segment tiles a launch of
     // their own, where closed rings are packed by corner.
     const long long units_all = (long long)p.TT * (p.SP + p.SS);
-    p.mixed = p.SP > 0 && p.SS > 0 && units_all < 4LL * sweep_blocks(grad, comp, p.stretch, false);
+    p.mixed = p.SP > 0 && p.SS > 0 && units_all < 4LL * sweep_blocks(grad, comp, p.stretch);
     plan(p.sk, p.SP, p.mixed ? p.SS : 0);
     plan(p.sks, 0, p.mixed ? 0 : p.SS);
     p.off_psrc = cv.take((size_t)p.SP * SRC_TILE * P_F4 * 16);
@@ -797,19 +991,57 @@ SweepPlan plan_sweep(int64_t n_tgt, int64_t n_src, int64_t m_seg, bool grad, boo
     p.off_ssrc = cv.take((size_t)p.SS * SRC_TILE * S_F4 * 16);
     p.off_sbox = cv.take((size_t)p.SS * 2 * 16);
     const size_t rows = (size_t)(comp ? 2 : 1) * p.ncomp;
-    if (p.sk.np + p.sk.ns > 0) p.off_part = cv.take((size_t)(p.sk.TT + p.sk.B) * rows * TGT_TILE * sizeof(float));
+    const long long units_p = (long long)p.TT * p.SP;
+    const bool far_size =
+        allow_far && (units_p >= FAR_MIN_UNITS || (n_tgt == n_src && grad && n_src >= FAR_SORT_MIN));
+    p.far = far_size && units_p <= FAR_MAX_UNITS;
+    if (!p.far && p.sk.np + p.sk.ns > 0) p.off_part = cv.take((size_t)(p.sk.TT + p.sk.B) * rows * TGT_TILE * sizeof(float));
     if (p.sks.ns > 0) p.off_part_s = cv.take((size_t)(p.sks.TT + p.sks.B) * rows * TGT_TILE * sizeof(float));
+    // Units on the tensor cores
+    if (far_size) {
+        p.KY = (p.SP + FAR_KCH - 1) / FAR_KCH;
+        const long long units = p.far ? units_p : FAR_MAX_UNITS;  // beyond the limit: keep the size monotone
+        p.B_near = sweep_blocks(grad, comp, p.stretch, SWEEP_NEAR);
+        p.B_far = (int)std::min<long long>(std::max(sm_count(), 1), units);
+        const size_t rows_f = (size_t)(comp ? 2 : 1) * (grad ? 14 : 3);
+        p.off_ftile = cv.take((size_t)p.SP * far_tile_bytes(grad));
+        p.off_fmask = cv.take((size_t)units * sizeof(unsigned));
+        p.off_fcnt = cv.take((size_t)p.TT * p.KY * (1 + FAR_GROUPS) * sizeof(int2));
+        p.off_nlist = cv.take((size_t)units * FAR_GROUPS * sizeof(uint2));
+        p.off_noff = cv.take(((size_t)p.TT * p.KY * FAR_GROUPS + 1) * sizeof(int2));
+        p.off_flist = cv.take((size_t)units * sizeof(uint2));
+        p.off_foff = cv.take(((size_t)p.TT * p.KY + 1) * sizeof(int2));
+        p.off_part_f = cv.take((size_t)(p.TT + p.B_far) * rows_f * TGT_TILE * sizeof(float));
+        constexpr int teams = Ring<SWEEP_NEAR>::TEAMS;
+        p.off_part_n = cv.take((size_t)(p.TT * FAR_GROUPS + p.B_near * teams) * rows * FAR_GROUP * sizeof(float));
+        if (n_tgt == n_src) {
+            const size_t n = (size_t)n_src;
+            const bool sortable = far_sort_bytes((int)n_src, &p.cub_bytes) == cudaSuccess;
+            p.sort = p.far && grad && sortable;
+            p.off_bnd = cv.take(FAR_BND_BLOCKS * 6 * sizeof(float));
+            p.off_key = cv.take(n * 4);
+            p.off_key2 = cv.take(n * 4);
+            p.off_idx = cv.take(n * 4);
+            p.off_perm = cv.take(n * 4);
+            p.off_cub = cv.take(p.cub_bytes);
+            p.off_spos = cv.take(n * 16);
+            p.off_sstr = cv.take(n * 16);
+            p.off_obox = cv.take((size_t)p.SP * 2 * 16);
+        }
+    }
     p.bytes = cv.off;
     return p;
 }
 
 template <bool G, bool C, bool S>
-static void launch_sweep(const SweepArgs& A, int B, bool segments, cudaStream_t st)
+static void launch_sweep(const SweepArgs& A, int B, int kind, cudaStream_t st)
 {
-    if (segments)
-        sweep_kernel<G, C, S, SWEEP_SEGMENTS><<<B, SWEEP_TPB, sweep_smem_bytes<G, C, S>(), st>>>(A);
+    if (kind == SWEEP_NEAR)
+        sweep_kernel<G, C, S, SWEEP_NEAR><<<B, SWEEP_TPB, sweep_smem_bytes<G, C, S, SWEEP_NEAR>(), st>>>(A);
+    else if (kind == SWEEP_SEGMENTS)
+        sweep_kernel<G, C, S, SWEEP_SEGMENTS><<<B, SWEEP_TPB, sweep_smem_bytes<G, C, S, SWEEP_SEGMENTS>(), st>>>(A);
     else
-        sweep_kernel<G, C, S, SWEEP_PARTICLES><<<B, SWEEP_TPB, sweep_smem_bytes<G, C, S>(), st>>>(A);
+        sweep_kernel<G, C, S, SWEEP_PARTICLES><<<B, SWEEP_TPB, sweep_smem_bytes<G, C, S, SWEEP_PARTICLES>(), st>>>(A);
 }
 
 cudaError_t run_sweep(const SweepPlan& p, char* ws, const float* tgt, const float* src_pos, const float* src_str,
@@ -823,11 +1055,27 @@ cudaError_t run_sweep(const SweepPlan& p, char* ws, const float* tgt, const floa
     float4* sbox = reinterpret_cast<float4*>(ws + p.off_sbox);
     float* part = reinterpret_cast<float*>(ws + p.off_part);
     float* part_s = reinterpret_cast<float*>(ws + p.off_part_s);
+    // Particles onto themselves are swept in curve order
+    const bool sorted = p.sort && tgt == src_pos;
+    const int* perm = nullptr;
+    float4* spos = reinterpret_cast<float4*>(ws + p.off_spos);
+    float4* sstr = reinterpret_cast<float4*>(ws + p.off_sstr);
+    if (sorted) {
+        const cudaError_t e = run_far_sort(p, ws, reinterpret_cast<const float4*>(src_pos), p.n_src, st);
+        if (e != cudaSuccess) return e;
+        perm = reinterpret_cast<const int*>(ws + p.off_perm);
+    }
     if (p.SP > 0) {
         trace_launch();
         pack_particles_kernel<<<p.SP, SRC_TILE, 0, st>>>(reinterpret_cast<const float4*>(src_pos),
-                                                         reinterpret_cast<const float4*>(src_str), p.n_src, psrc,
-                                                         pbox);
+                                                         reinterpret_cast<const float4*>(src_str), p.n_src, perm, spos,
+                                                         sstr, psrc, pbox);
+    }
+    const float* own = out.str;
+    if (sorted) {
+        tgt = src_pos = reinterpret_cast<const float*>(spos);
+        src_str = reinterpret_cast<const float*>(sstr);
+        own = src_str;
     }
     if (p.SS > 0) {
         trace_launch();
@@ -836,12 +1084,40 @@ cudaError_t run_sweep(const SweepPlan& p, char* ws, const float* tgt, const floa
                                                         vatistas_n, p.mixed ? 0 : 1, ssrc, sbox);
     }
     int* err = dev_err_ptr();
+    UnitList uln{}, ulf{};
+    const unsigned char* ftile = reinterpret_cast<const unsigned char*>(ws + p.off_ftile);
+    if (p.far) {
+        auto list = [&](size_t l, size_t o, int T, int B, int max_cost) {
+            UnitList u;
+            u.list = reinterpret_cast<const uint2*>(ws + l);
+            u.off = reinterpret_cast<const int2*>(ws + o);
+            u.TT = T;
+            u.KY = p.KY;
+            u.B = B;
+            u.max_cost = max_cost;
+            return u;
+        };
+        uln = list(p.off_nlist, p.off_noff, p.TT * FAR_GROUPS, p.B_near * Ring<SWEEP_NEAR>::TEAMS,
+                   Ring<SWEEP_NEAR>::WARPS * NEAR_COST);
+        ulf = list(p.off_flist, p.off_foff, p.TT, p.B_far, FAR_GROUPS);
+        cudaError_t e = run_far_pack(reinterpret_cast<const float4*>(src_pos), reinterpret_cast<const float4*>(src_str),
+                                     p.n_src, pbox, p.SP, p.grad, reinterpret_cast<unsigned char*>(ws + p.off_ftile), st);
+        if (e == cudaSuccess)
+            e = run_far_lists(reinterpret_cast<const float4*>(tgt), p.n_tgt, ftile, p.SP, p.TT, p.grad, pbox,
+                              (float)((double)RHO_FAR * RHO_FAR * (double)sigma * (double)sigma),
+                              reinterpret_cast<unsigned*>(ws + p.off_fmask),
+                              reinterpret_cast<int2*>(ws + p.off_fcnt), reinterpret_cast<uint2*>(ws + p.off_nlist),
+                              reinterpret_cast<int2*>(ws + p.off_noff), reinterpret_cast<uint2*>(ws + p.off_flist),
+                              reinterpret_cast<int2*>(ws + p.off_foff), st);
+        if (e != cudaSuccess) return e;
+    }
     if (p.SP + p.SS > 0) {
-        if (p.sk.np + p.sk.ns > 0) blocks_per_sm(p.grad, p.comp, p.stretch, false);  // shared-memory opt-in
-        if (p.sks.ns > 0) blocks_per_sm(p.grad, p.comp, p.stretch, true);
+        // shared-memory opt-in
+        if (p.sk.np + p.sk.ns > 0) blocks_per_sm(p.grad, p.comp, p.stretch, p.far ? SWEEP_NEAR : SWEEP_PARTICLES);
+        if (p.sks.ns > 0) blocks_per_sm(p.grad, p.comp, p.stretch, SWEEP_SEGMENTS);
         SweepArgs A;
         A.tgt = reinterpret_cast<const float4*>(tgt);
-        A.tstr = p.stretch ? reinterpret_cast<const float4*>(out.str) : nullptr;
+        A.tstr = p.stretch ? reinterpret_cast<const float4*>(own) : nullptr;
         A.n_tgt = p.n_tgt;
         A.psrc = psrc;
         A.pbox = pbox;
@@ -864,37 +1140,64 @@ cudaError_t run_sweep(const SweepPlan& p, char* ws, const float* tgt, const floa
             TraceScope ts(seg ? VPM_TRACE_SEGMENTS : p.grad ? VPM_TRACE_SWEEP : VPM_TRACE_SWEEP_VEL, st);
             A.sk = seg ? p.sks : p.sk;
             A.part = seg ? part_s : part;
-            const int B = A.sk.B;
+            const int B = !seg && p.far ? p.B_near : A.sk.B;
+            const int k = seg ? SWEEP_SEGMENTS : p.far ? SWEEP_NEAR : SWEEP_PARTICLES;
+            if (k == SWEEP_NEAR) {
+                A.ul = uln;
+                A.part = reinterpret_cast<float*>(ws + p.off_part_n);
+                FarArgs F;
+                F.tgt = A.tgt;
+                F.n_tgt = p.n_tgt;
+                F.tiles = ftile;
+                F.ul = ulf;
+                F.part = reinterpret_cast<float*>(ws + p.off_part_f);
+                F.dev_err = err;
+                trace_launch();
+                const cudaError_t e = run_far_sweep(F, p.grad, p.comp, st);
+                if (e != cudaSuccess) return e;
+            }
             if (p.grad && p.stretch) {
                 if (p.comp)
-                    launch_sweep<true, true, true>(A, B, seg, st);
+                    launch_sweep<true, true, true>(A, B, k, st);
                 else
-                    launch_sweep<true, false, true>(A, B, seg, st);
+                    launch_sweep<true, false, true>(A, B, k, st);
             } else if (p.grad) {
                 if (p.comp)
-                    launch_sweep<true, true, false>(A, B, seg, st);
+                    launch_sweep<true, true, false>(A, B, k, st);
                 else
-                    launch_sweep<true, false, false>(A, B, seg, st);
+                    launch_sweep<true, false, false>(A, B, k, st);
             } else {
                 if (p.comp)
-                    launch_sweep<false, true, false>(A, B, seg, st);
+                    launch_sweep<false, true, false>(A, B, k, st);
                 else
-                    launch_sweep<false, false, false>(A, B, seg, st);
+                    launch_sweep<false, false, false>(A, B, k, st);
             }
         }
     }
     EpiArgs E;
     E.sk = p.sk;
-    E.part = part;
+    E.part = p.far ? reinterpret_cast<const float*>(ws + p.off_part_n) : part;
     E.sks = p.sks;
     E.part_s = part_s;
+    E.far = p.far ? 1 : 0;
+    E.uln = uln;
+    E.ulf = ulf;
+    E.part_f = reinterpret_cast<const float*>(ws + p.off_part_f);
+    E.ncomp_f = p.grad ? 14 : 3;
     E.n = p.n_tgt;
     E.ncomp = p.ncomp;
     E.comp = p.comp ? 1 : 0;
     E.o = out;
+    E.o.str = own;
+    E.perm = perm;
     E.dev_err = err;
     trace_launch();
-    epilogue_kernel<<<(p.n_tgt + 255) / 256, 256, 0, st>>>(E);
+    // Threads per target: enough to give every SM a few blocks
+    const long long want = 4LL * 256 * std::max(sm_count(), 1);
+    if (2LL * p.n_tgt <= want)
+        epilogue_kernel<8><<<(p.n_tgt + 31) / 32, 256, 0, st>>>(E);
+    else
+        epilogue_kernel<1><<<(p.n_tgt + 255) / 256, 256, 0, st>>>(E);
     return cudaGetLastError();
 }
 
@@ -902,14 +1205,20 @@ cudaError_t run_pse(const SweepPlan& p, char* ws, const float* pos, const float*
                     float sigma, float nu, float* dGdt, cudaStream_t st)
 {
     if (n == 0) return cudaSuccess;
-    const float4* pbox = reinterpret_cast<const float4*>(ws + p.off_pbox);
+    // the exchange takes the particles in the caller's order
+    const float4* pbox = reinterpret_cast<const float4*>(ws + (p.sort ? p.off_obox : p.off_pbox));
     const double s = sigma;
     const float inv2s2 = (float)(0.5 / (s * s));
     const float cut2 = (float)((double)RHO_FAR * RHO_FAR * s * s);
     // (2/sigma^2) (2 pi sigma^2)^(-3/2)
     const float pref = (float)(2.0 / (s * s) * pow(2.0 * 3.14159265358979323846 * s * s, -1.5));
+    if (p.sort) {
+        trace_launch();
+        tile_box_kernel<<<p.SP, SRC_TILE, 0, st>>>(reinterpret_cast<const float4*>(pos), n,
+                                                   reinterpret_cast<float4*>(ws + p.off_obox));
+    }
     TraceScope ts(VPM_TRACE_PSE, st);
-    pse_kernel<<<(n + 64 * PSE_W - 1) / (64 * PSE_W), PSE_T, 0, st>>>(reinterpret_cast<const float4*>(pos),
+    pse_kernel<<<(n + 63) / 64, PSE_T, 0, st>>>(reinterpret_cast<const float4*>(pos),
                                                           reinterpret_cast<const float4*>(str), nu_t, n, pbox, p.SP,
                                                           inv2s2, cut2, nu, pref, dGdt);
     return cudaGetLastError();
