@@ -127,8 +127,9 @@ __device__ __forceinline__ void far_weight(f2 t, uint32_t& hi, uint32_t& neg)
 // 8 bits per axis: three radix passes, and cells far smaller than a tile.
 // ---------------------------------------------------------------------------
 constexpr int CURVE_BITS = 8;
+constexpr int CURVE_BND_BLOCKS = 128;  // partial boxes of the curve's bounding cube
 
-__global__ void __launch_bounds__(256) far_bounds_kernel(const float4* __restrict__ pos, int n, float* __restrict__ bnd)
+__global__ void __launch_bounds__(256) curve_bounds_kernel(const float4* __restrict__ pos, int n, float* __restrict__ bnd)
 {
     float v[6] = {INFINITY, INFINITY, INFINITY, INFINITY, INFINITY, INFINITY};  // least of x and of -x
     for (int i = blockIdx.x * 256 + threadIdx.x; i < n; i += gridDim.x * 256) {
@@ -183,7 +184,7 @@ __device__ __forceinline__ unsigned hilbert_key(unsigned x, unsigned y, unsigned
     return k;
 }
 
-__global__ void __launch_bounds__(256) far_keys_kernel(const float4* __restrict__ pos, int n,
+__global__ void __launch_bounds__(256) curve_keys_kernel(const float4* __restrict__ pos, int n,
                                                        const float* __restrict__ bnd, int nb,
                                                        unsigned* __restrict__ key, int* __restrict__ idx)
 {
@@ -209,27 +210,34 @@ __global__ void __launch_bounds__(256) far_keys_kernel(const float4* __restrict_
     idx[i] = i;
 }
 
-cudaError_t far_sort_bytes(int n, size_t* bytes)
+bool curve_layout(int64_t n, Carve& cv, CurveWs& w)
 {
-    *bytes = 0;
-    return cub::DeviceRadixSort::SortPairs(nullptr, *bytes, (const unsigned*)nullptr, (unsigned*)nullptr,
-                                           (const int*)nullptr, (int*)nullptr, n, 0, 3 * CURVE_BITS);
+    const bool ok = cub::DeviceRadixSort::SortPairs(nullptr, w.cub_bytes, (const unsigned*)nullptr, (unsigned*)nullptr,
+                                                    (const int*)nullptr, (int*)nullptr, (int)n, 0,
+                                                    3 * CURVE_BITS) == cudaSuccess;
+    w.bnd = cv.take(CURVE_BND_BLOCKS * 6 * sizeof(float));
+    w.key = cv.take((size_t)n * 4);
+    w.key2 = cv.take((size_t)n * 4);
+    w.idx = cv.take((size_t)n * 4);
+    w.perm = cv.take((size_t)n * 4);
+    w.cub = cv.take(w.cub_bytes);
+    return ok;
 }
 
-cudaError_t run_far_sort(const SweepPlan& p, char* ws, const float4* pos, int n, cudaStream_t st)
+cudaError_t run_curve_sort(const CurveWs& w, char* ws, const float4* pos, int n, cudaStream_t st)
 {
-    float* bnd = reinterpret_cast<float*>(ws + p.off_bnd);
-    unsigned* key = reinterpret_cast<unsigned*>(ws + p.off_key);
-    unsigned* key2 = reinterpret_cast<unsigned*>(ws + p.off_key2);
-    int* idx = reinterpret_cast<int*>(ws + p.off_idx);
-    int* perm = reinterpret_cast<int*>(ws + p.off_perm);
-    const int nb = std::min(FAR_BND_BLOCKS, (n + 255) / 256);
+    float* bnd = reinterpret_cast<float*>(ws + w.bnd);
+    unsigned* key = reinterpret_cast<unsigned*>(ws + w.key);
+    unsigned* key2 = reinterpret_cast<unsigned*>(ws + w.key2);
+    int* idx = reinterpret_cast<int*>(ws + w.idx);
+    int* perm = reinterpret_cast<int*>(ws + w.perm);
+    const int nb = std::min(CURVE_BND_BLOCKS, (n + 255) / 256);
     trace_launch(2);
-    far_bounds_kernel<<<nb, 256, 0, st>>>(pos, n, bnd);
-    far_keys_kernel<<<(n + 255) / 256, 256, 0, st>>>(pos, n, bnd, nb, key, idx);
-    size_t bytes = p.cub_bytes;
-    const cudaError_t e = cub::DeviceRadixSort::SortPairs(ws + p.off_cub, bytes, key, key2, idx, perm, n, 0,
-                                                          3 * CURVE_BITS, st);
+    curve_bounds_kernel<<<nb, 256, 0, st>>>(pos, n, bnd);
+    curve_keys_kernel<<<(n + 255) / 256, 256, 0, st>>>(pos, n, bnd, nb, key, idx);
+    size_t bytes = w.cub_bytes;
+    const cudaError_t e =
+        cub::DeviceRadixSort::SortPairs(ws + w.cub, bytes, key, key2, idx, perm, n, 0, 3 * CURVE_BITS, st);
     return e != cudaSuccess ? e : cudaGetLastError();
 }
 

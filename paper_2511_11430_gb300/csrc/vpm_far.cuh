@@ -60,7 +60,6 @@ constexpr long long FAR_MAX_UNITS = 1LL << 26;   // ... and to which (the unit l
 // side of the BVI wake: 16,000 particles 819 us without and 744 us with it, 12,000 particles
 // 611 and 638 us; hover wake 679 and 690 us, 488 and 572 us).
 constexpr int FAR_SORT_MIN = 16384;
-constexpr int FAR_BND_BLOCKS = 128;              // partial boxes of the curve's bounding cube
 constexpr int FAR_KCH = 2048;                    // source tiles per block of the mask and list kernels
 constexpr float FAR_FSCALE = 256.f;              // features are scaled by this before their FP16 split
 
@@ -140,9 +139,6 @@ struct FarArgs {
     int* dev_err;
 };
 
-// Hilbert-curve order of n particles (sorted position -> index, in SweepPlan::off_perm).
-cudaError_t far_sort_bytes(int n, size_t* bytes);
-cudaError_t run_far_sort(const SweepPlan& p, char* ws, const float4* pos, int n, cudaStream_t st);
 cudaError_t run_far_pack(const float4* pos, const float4* str, int n, const float4* box, int SP, bool grad,
                          unsigned char* tiles, cudaStream_t st);
 cudaError_t run_far_lists(const float4* tgt, int n_tgt, const unsigned char* tiles, int SP, int TT, bool grad,

@@ -39,6 +39,14 @@ int* dev_err_ptr();          // device error word of the current device
 int sweep_blocks(bool grad, bool comp, bool stretch, int kind = 0);  // resident sweep blocks (current device)
 int adjoint_blocks(bool comp);
 
+// Workspace of the curve order of n particles (offsets).
+struct CurveWs {
+    size_t bnd = 0, key = 0, key2 = 0, idx = 0, perm = 0, cub = 0, cub_bytes = 0;
+};
+bool curve_layout(int64_t n, Carve& cv, CurveWs& w);  // false: the sort's scratch size could not be had
+// Hilbert-curve order of n particles: sorted position -> index in ws + w.perm.
+cudaError_t run_curve_sort(const CurveWs& w, char* ws, const float4* pos, int n, cudaStream_t st);
+
 struct SweepPlan {
     int n_tgt = 0, n_src = 0, m_seg = 0;
     int TT = 0, SP = 0, SS = 0;
@@ -54,8 +62,8 @@ struct SweepPlan {
     size_t off_psrc = 0, off_pbox = 0, off_ssrc = 0, off_sbox = 0, off_part = 0, off_part_s = 0, bytes = 0;
     // Particles onto themselves: the particles are put in Hilbert-curve order first
     bool sort = false;
-    size_t off_bnd = 0, off_key = 0, off_key2 = 0, off_idx = 0, off_perm = 0, off_cub = 0, cub_bytes = 0, off_spos = 0,
-           off_sstr = 0, off_obox = 0;
+    CurveWs curve{};
+    size_t off_spos = 0, off_sstr = 0, off_obox = 0;
     size_t off_ftile = 0, off_fmask = 0, off_fcnt = 0, off_nlist = 0, off_noff = 0, off_flist = 0, off_foff = 0,
            off_part_f = 0, off_part_n = 0;
 };
@@ -88,6 +96,12 @@ cudaError_t run_sweep(const SweepPlan& p, char* ws, const float* tgt, const floa
 // Particle strength exchange added into dGdt (uses the particle tile boxes of the plan).
 cudaError_t run_pse(const SweepPlan& p, char* ws, const float* pos, const float* str, const float* nu_t, int n,
                     float sigma, float nu, float* dGdt, cudaStream_t st);
+
+// The same over n particles in the order pos, str, nu_t have; particle i's term goes to dGdt
+// element perm[i] (perm null: i).  box: room for the tile boxes (pse_box_bytes).
+size_t pse_box_bytes(int64_t n);
+cudaError_t run_pse_sorted(const float4* pos, const float4* str, const float* nu_t, const int* perm, float4* box, int n,
+                           float sigma, float nu, float* dGdt, cudaStream_t st);
 
 // Time step kernels.
 cudaError_t run_cast_state(const double* x, const double* G, const float* vol, int n, float* pos, float* str,
@@ -127,7 +141,8 @@ vpm_status run_wake_convert_row(const double* U, const double* D, const double* 
                                 cudaStream_t st, const char** msg);
 cudaError_t tree_workspace(long long n, size_t* bytes);
 struct TreeRhsWs {
-    size_t tree, stree, up, Jp, sp, sg, nut, counter, bytes;
+    size_t tree, stree, up, Jp, sp, sg, snut, nut, box, bytes;
+    CurveWs curve;
 };
 // A built segment tree, as the treecode's traversal reads it.
 struct SegTreeView {
