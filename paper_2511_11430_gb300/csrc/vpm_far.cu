@@ -363,6 +363,14 @@ constexpr int LIST_TPB = SWEEP_TPB;
 // group's cost in the pair sweep.
 __device__ __forceinline__ int near_cost(unsigned m, int g) { return (m >> (8 + 6 * g)) & 63u; }
 
+// A unit's cost in the tensor-core sweep: a lone warpgroup runs at less than half the rate
+// of four, so the first group costs as much as the other three.
+__device__ __forceinline__ int far_cost(unsigned m)
+{
+    const int c = __popc(m & FAR_ALL);
+    return c ? FAR_COST_FIRST + c - 1 : 0;
+}
+
 // cnt[0 .. TT KY): (units, cost) of the tensor-core list by (target tile, chunk); then the
 // pair sweep's by (target tile, group, chunk).
 template <bool GRAD>
@@ -407,18 +415,19 @@ __global__ void __launch_bounds__(LIST_TPB) far_mask_kernel(const float4* __rest
                     const float dz = fmaxf(0.f, fmaxf(c.z - lo[5], lo[2] - c.z));
                     far = far && dx * dx + dy * dy + dz * dz > need2;
                 }
-            // (a group wholly past the last target counts as far: the pair sweep has nothing to do there)
             int cn = 0;
-            if (far)
+            if (t * TGT_TILE + g * FAR_GROUP >= n_tgt)
+                ;  // no target: in neither list
+            else if (far)
                 m |= 1u << g;
             else
 #pragma unroll 1
                 for (int w = g * GW; w < (g + 1) * GW; ++w) cn += boxes_near(wbox[w], tlo, thi, far2) ? NEAR_COST : 1;
             m |= (unsigned)cn << (8 + 6 * g);
-            v[1 + g][0] += !far, v[1 + g][1] += cn;
+            v[1 + g][0] += cn != 0, v[1 + g][1] += cn;
         }
         mask[(size_t)t * SP + k] = m;
-        const int c1 = __popc(m & FAR_ALL);
+        const int c1 = far_cost(m);
         v[0][0] += c1 != 0, v[0][1] += c1;
     }
 #pragma unroll
@@ -485,9 +494,9 @@ __global__ void __launch_bounds__(LIST_TPB) far_emit_kernel(const unsigned* __re
     const unsigned lt = (1u << lane) - 1u;
     for (int ks = k0; ks < k1; ks += LIST_TPB) {
         const int k = ks + threadIdx.x;
-        const unsigned m = k < k1 ? mask[(size_t)t * SP + k] : g < 0 ? 0u : FAR_ALL;
-        const bool in = g < 0 ? (m & FAR_ALL) != 0u : !((m >> g) & 1u);
-        const int c = !in ? 0 : g < 0 ? __popc(m & FAR_ALL) : near_cost(m, g);
+        const unsigned m = k < k1 ? mask[(size_t)t * SP + k] : 0u;
+        const int c = g < 0 ? far_cost(m) : near_cost(m, g);
+        const bool in = c != 0;
         const unsigned q = __ballot_sync(0xffffffffu, in);
         int s = c;  // costs up to this lane
 #pragma unroll

@@ -44,6 +44,7 @@ constexpr int FAR_GROUPS = TGT_TILE / FAR_GROUP; // groups of a target tile
 constexpr unsigned FAR_ALL = (1u << FAR_GROUPS) - 1u;
 // Cost in the pair sweep of a warp's tile within 7 sigma, against one of a tile beyond.
 constexpr int NEAR_COST = 3;
+constexpr int FAR_COST_FIRST = 3;                // cost of a far unit's first group, against one of each further
 // Acceptance ratio.  The error does not depend on it where it was measured (0.2 to 0.6: u
 // 1.31e-7 to 1.34e-7, grad u 1.83e-7 throughout on the 100,000-particle hover wake, whose
 // error comes from the near pairs), since every pair is evaluated at any ratio; beyond 0.5
@@ -77,9 +78,11 @@ struct FarTile {
 constexpr size_t far_tile_bytes(bool grad) { return grad ? FarTile<true>::BYTES : FarTile<false>::BYTES; }
 
 // A list of units ordered by target tile: (source tile << 4 | group mask, cost of the
-// units before it); the pair sweep's is ordered by group and holds the source tile alone.  A unit's cost is the number of its groups in the tensor-core list; in
-// the pair sweep's the number of the group's warps, those within 7 sigma counted NEAR_COST times.  The cost line is cut into equal ranges, one per block (at most B of them, and
-// at least a whole unit long, so that every range holds the start of one); block b runs the
+// units before it); the pair sweep's is ordered by group and holds the source tile alone.
+// A unit's cost in the tensor-core list is far_cost of its groups, in the pair sweep's the
+// number of the group's warps, those within 7 sigma counted NEAR_COST times.  The cost line
+// is cut into equal ranges, one per block or team (at most B of them, and at least a whole
+// unit long, so that every range holds the start of one); block b runs the
 // units whose cost starts in its range and writes one partial sum per target tile into
 // slot b + t.
 struct UnitList {

@@ -53,6 +53,7 @@ struct SweepPlan {
     bool grad = false, comp = false;
     bool stretch = false;  // accumulate the transposed stretching J^T Gamma_i per target
     int ncomp = 0;         // logical accumulator rows (3, 14 or 17)
+    int kind = 0, kind_s = 0;  // sweep kernels of the particle tiles (without the tensor cores) and the segment tiles
     bool mixed = false;  // particle and segment tiles in one launch (small problems)
     StreamK sk{};        // particle tiles, and the segment tiles when mixed (one launch)
     StreamK sks{};       // otherwise the segment tiles (a launch of their own)

@@ -32,6 +32,7 @@
 
 #include <algorithm>
 #include <mutex>
+#include <type_traits>
 
 #include "vpm_common.cuh"
 #include "vpm_far.cuh"
@@ -63,10 +64,10 @@ __device__ __forceinline__ void particle_subset(Acc<GRAD, STRETCH>& a, const flo
                                                 f2 Y, f2 Z, const NearConst& nc, const Own& o)
 {
 #pragma unroll 1
-    for (int h = 0; h < SRC_TILE / 32; ++h) {
+    for (int h = 0; 32 * h < cnt; ++h) {
         unsigned m = h == 0 ? keep[0] : h == 1 ? keep[1] : h == 2 ? keep[2] : keep[3];
         const int left = cnt - 32 * h;
-        if (invert) m = ~m & (left >= 32 ? 0xffffffffu : left > 0 ? (1u << left) - 1u : 0u);
+        if (invert) m = ~m & (left >= 32 ? 0xffffffffu : (1u << left) - 1u);
         for (const float4* sh = s + 32 * h * P_F4; m; m &= m - 1)
             particle_source<GRAD, STRETCH, NEAR>(a, sh + (__ffs(m) - 1) * P_F4, X, Y, Z, nc, o);
     }
@@ -283,19 +284,35 @@ __host__ __device__ constexpr int n_rows()
 // (256-target group, source tile) units: with blocks of 1,024 targets three quarters of
 // the warps had nothing to do.  (Measured: the particle launch compiled
 // without its segment loop is allocated fewer registers and runs 4% slower.)
-constexpr int SWEEP_PARTICLES = 0, SWEEP_SEGMENTS = 1, SWEEP_NEAR = 2;
-constexpr int SWEEP_KINDS = 3;
+constexpr int SWEEP_PARTICLES = 0, SWEEP_SEGMENTS = 1, SWEEP_NEAR = 2, SWEEP_SMALL = 3, SWEEP_SEG_SMALL = 4;
+constexpr int SWEEP_KINDS = 5;
 
-// A ring of source stages serves a team of warps: the whole block, or with SWEEP_NEAR
-// each warpgroup its own.
+// A ring of source stages serves a team of warps: the whole block, or each warpgroup its
+// own.  Teams of four warps make finer work units (256 targets instead of 1,024, and with
+// half tiles 64 sources): a small problem then reaches every SM, and a few targets or a few
+// waves of units leave less idle.  (2,000 particles and 640 segments: 42 units of
+// 1,024 x 128, 73 us.)
+// Units (1,024 targets x 128 sources) below which teams sweep the particle tiles, and the
+// segment tiles (whose loop pays more for the folds after half tiles: 5,120 segments onto
+// 100,000 particles 1.25 ms with whole blocks and tiles, 1.43 ms with teams; onto 20,000, 5.3
+// units a block, 317 and 324 us).
+constexpr long long SMALL_MAX_UNITS = 16384, SEG_SMALL_MAX_UNITS = 512;
+// Segment tiles up to which a small problem sweeps them, one segment at a time, with its
+// particle tiles.
+constexpr int MIXED_MAX_TILES = 8;
+
 template <int KIND>
 struct Ring {
     static constexpr bool LIST = KIND == SWEEP_NEAR;
-    static constexpr int TEAMS = LIST ? SWEEP_CW / 4 : 1, WARPS = SWEEP_CW / TEAMS;
-    static constexpr int STAGES = LIST ? 2 : SWEEP_STAGES;         // per team
-    static constexpr int BOX = SRC_TILE * (LIST ? P_F4 : S_F4);    // the tile's bounding box, float4s into a stage
+    static constexpr int TEAMS = KIND == SWEEP_PARTICLES || KIND == SWEEP_SEGMENTS ? 1 : SWEEP_CW / 4;
+    static constexpr int WARPS = SWEEP_CW / TEAMS;
+    static constexpr bool SEG = KIND == SWEEP_SEGMENTS || KIND == SWEEP_SEG_SMALL;
+    static constexpr int UNIT = KIND == SWEEP_SMALL || KIND == SWEEP_SEG_SMALL ? SRC_TILE / 2 : SRC_TILE;  // sources
+    static constexpr int PER_TILE = SRC_TILE / UNIT;
+    static constexpr int STAGES = TEAMS > 1 ? 2 : SWEEP_STAGES;  // per team
+    static constexpr int BOX = UNIT * (LIST ? P_F4 : S_F4);      // the tile's bounding box, float4s into a stage
     static constexpr int F4 = BOX + 2;
-    static constexpr int TGT = LIST ? FAR_GROUP : TGT_TILE;        // targets of a team
+    static constexpr int TGT = WARPS * 64;                       // targets of a team
 };
 
 // Dynamic shared memory: the source stages, then the running sums of the consumer
@@ -327,7 +344,9 @@ __global__ void __launch_bounds__(SWEEP_TPB, 1) sweep_kernel(const SweepArgs A)
 
     const StreamK& sk = A.sk;
     const UnitList& ul = A.ul;
-    const int b = blockIdx.x * R::TEAMS + team;
+    // teams of different blocks first, so that few teams spread over the SMs
+    const int b = team * gridDim.x + blockIdx.x;
+    bool mine = true;      // the team has a unit
     long long lo_b, hi_b;  // this team's range: of the cost line, or of the list's entries
     int t0, k0;
     if constexpr (LIST) {
@@ -340,10 +359,11 @@ __global__ void __launch_bounds__(SWEEP_TPB, 1) sweep_kernel(const SweepArgs A)
         __syncthreads();
         lo_b = range_s[team][0], hi_b = range_s[team][1], t0 = range_s[team][2];
         k0 = 0;
+        mine = lo_b < hi_b;
     } else {
-        lo_b = sk.lo(b), hi_b = sk.lo(b + 1);
+        lo_b = sk.lo(min(b, sk.B)), hi_b = sk.lo(min(b + 1, sk.B));
         sk.first_at_or_after(lo_b, t0, k0);
-        if (t0 >= sk.TT || sk.unit_start(t0, k0) >= hi_b) return;  // block owns no unit (uniform)
+        mine = t0 < sk.TT && sk.unit_start(t0, k0) < hi_b;
     }
     const int nunits = sk.np + sk.ns;
 
@@ -352,15 +372,15 @@ __global__ void __launch_bounds__(SWEEP_TPB, 1) sweep_kernel(const SweepArgs A)
         issued_round[s] = round;
         fence_proxy_async_smem();
         if (LIST || kk < sk.np) {
-            const uint32_t bytes = SRC_TILE * P_F4 * 16;
+            const uint32_t bytes = R::UNIT * P_F4 * 16;
             mbar_expect_tx(&full[s], bytes + 32);
-            bulk_g2s(stage + (size_t)s * R::F4, A.psrc + (size_t)kk * SRC_TILE * P_F4, bytes, &full[s]);
-            bulk_g2s(stage + (size_t)s * R::F4 + R::BOX, A.pbox + 2 * kk, 32, &full[s]);
+            bulk_g2s(stage + (size_t)s * R::F4, A.psrc + (size_t)kk * R::UNIT * P_F4, bytes, &full[s]);
+            bulk_g2s(stage + (size_t)s * R::F4 + R::BOX, A.pbox + 2 * (kk / R::PER_TILE), 32, &full[s]);
         } else {
-            const uint32_t bytes = SRC_TILE * S_F4 * 16;
+            const uint32_t bytes = R::UNIT * S_F4 * 16;
             mbar_expect_tx(&full[s], bytes + 32);
-            bulk_g2s(stage + (size_t)s * R::F4, A.ssrc + (size_t)(kk - sk.np) * SRC_TILE * S_F4, bytes, &full[s]);
-            bulk_g2s(stage + (size_t)s * R::F4 + R::BOX, A.sbox + 2 * (kk - sk.np), 32, &full[s]);
+            bulk_g2s(stage + (size_t)s * R::F4, A.ssrc + (size_t)(kk - sk.np) * R::UNIT * S_F4, bytes, &full[s]);
+            bulk_g2s(stage + (size_t)s * R::F4 + R::BOX, A.sbox + 2 * ((kk - sk.np) / R::PER_TILE), 32, &full[s]);
         }
     };
     // The unit `ahead` places after the i-th, (t, k), in this team's run, if the team owns it.
@@ -384,14 +404,14 @@ __global__ void __launch_bounds__(SWEEP_TPB, 1) sweep_kernel(const SweepArgs A)
             issued_round[s0 + s] = -1;
         }
         mbar_fence_init();
-        for (int s = 0; s < R::STAGES; ++s) {  // first fill of the ring
+        for (int s = 0; mine && s < R::STAGES; ++s) {  // first fill of the ring
             int kk;
             if (!unit_ahead(0, t0, k0, s, kk)) break;
             issue(kk, s0 + s, 0);
         }
     }
     __syncthreads();
-    if (LIST && lo_b >= hi_b) return;  // team owns no unit
+    if (!mine) return;  // the team owns no unit
 
     // ---------------- consumers ----------------
     const int ct = warp * 32 + lane;  // consumer thread index
@@ -452,8 +472,8 @@ __global__ void __launch_bounds__(SWEEP_TPB, 1) sweep_kernel(const SweepArgs A)
         // stretching from the tile's sums afterwards.  Near particle tiles accumulate the
         // stretching pair by pair (it cancels there) with the strengths loaded for them.
         const int ti0 = t * R::TGT + (warp % R::WARPS) * 64 + lane, ti1 = ti0 + 32;
-        if (LIST || (KIND == SWEEP_PARTICLES && k < sk.np)) {
-            const int cnt = min(SRC_TILE, A.n_src - k * SRC_TILE);
+        if (LIST || (!R::SEG && k < sk.np)) {
+            const int cnt = min(R::UNIT, A.n_src - k * R::UNIT);  // (the last half tile may be empty)
             const float4 tlo = src[R::BOX], thi = src[R::BOX + 1];
             if (boxes_near(wbox[warp], tlo, thi, A.nc.far2)) {
                 Own own{zero2(), zero2(), zero2()};
@@ -467,9 +487,9 @@ __global__ void __launch_bounds__(SWEEP_TPB, 1) sweep_kernel(const SweepArgs A)
                 }
                 // Sources at least 7 sigma from both of the warp's boxes take the point-vortex
                 // form (and give their stretching from their sums, as a far tile does)
-                unsigned keep[SRC_TILE / 32];
+                unsigned keep[SRC_TILE / 32] = {};
 #pragma unroll
-                for (int h = 0; h < SRC_TILE / 32; ++h) {
+                for (int h = 0; h < R::UNIT / 32; ++h) {
                     const int j = 32 * h + lane;
                     const float4 q0 = src[j * P_F4], q1 = src[j * P_F4 + 1];
                     const float4 pt = make_float4(-q0.x, -q0.z, -q1.x, 0.f);
@@ -489,13 +509,13 @@ __global__ void __launch_bounds__(SWEEP_TPB, 1) sweep_kernel(const SweepArgs A)
                 finish_tile<GRAD, STRETCH>(acc, tf, A.tstr, ti0, ti1, A.n_tgt);
             }
         } else {
-            const int cnt = min(SRC_TILE, A.m_seg - (k - sk.np) * SRC_TILE);
+            const int cnt = min(R::UNIT, A.m_seg - (k - sk.np) * R::UNIT);
             const float4 tlo = src[R::BOX], thi = src[R::BOX + 1];
             const float margin = 1e-3f * tlo.w;
             const bool safe = A.core_pos && margin > 0.f && !boxes_near(wbox[warp], tlo, thi, margin * margin);
             Acc<GRAD, false> tf;
             tf.zero();
-            if (KIND == SWEEP_SEGMENTS && thi.w != 0.f) {  // closed four-sided rings, packed by corner
+            if (R::SEG && thi.w != 0.f) {  // closed four-sided rings, packed by corner
                 if (safe)
                     ring_tile<GRAD, true>(tf, src, cnt >> 2, X, Y, Z, A.vn);
                 else
@@ -554,6 +574,7 @@ struct EpiArgs {
     StreamK sk, sks;  // the particle and the segment launch
     const float* part;
     const float* part_s;
+    int tgt, tgt_s;     // targets per partial sum of the two launches
     int far;            // the particle units are split between two lists
     UnitList uln, ulf;  // ... those of the particle launch and of the tensor-core launch
     const float* part_f;
@@ -580,7 +601,6 @@ __global__ void __launch_bounds__(256) epilogue_kernel(const EpiArgs E)
     const int part_i = threadIdx.x / TB;
     const int i = blockIdx.x * TB + threadIdx.x % TB;
     if (PARTS == 1 && i >= E.n) return;
-    const int t = min(i, E.n - 1) / TGT_TILE, l = i % TGT_TILE;
     // The partial sums are folded in FP32 double-float arithmetic (hi by Knuth's
     // two-sum, the low words added apart: about 48 bits) and converted to FP64 once
     // per row; the FP64 pipe, a small fraction of the FP32 rate here, keeps only the
@@ -588,7 +608,12 @@ __global__ void __launch_bounds__(256) epilogue_kernel(const EpiArgs E)
     float H[17], Lw[17];
 #pragma unroll
     for (int c = 0; c < 17; ++c) H[c] = 0.f, Lw[c] = 0.f;
-    auto add = [&](const float* P, int ncomp, int ld) {
+    // ld: targets per partial sum, a constant
+    using Whole = std::integral_constant<int, TGT_TILE>;
+    using Team = std::integral_constant<int, FAR_GROUP>;
+    static_assert(FAR_GROUP == Ring<SWEEP_SMALL>::TGT, "targets of a team");
+    auto add = [&](const float* P, int ncomp, auto ldc) {
+        constexpr int ld = decltype(ldc)::value;
 #pragma unroll
         for (int c = 0; c < 17; ++c) {  // a constant bound keeps the sums in registers
             if (c < ncomp) {
@@ -600,16 +625,17 @@ __global__ void __launch_bounds__(256) epilogue_kernel(const EpiArgs E)
             }
         }
     };
-    auto add_list = [&](const UnitList& ul, const float* part, int ncomp, int ld) {  // ld targets per list row
+    auto add_list = [&](const UnitList& ul, const float* part, int ncomp, auto ldc) {
+        constexpr int ld = decltype(ldc)::value;
         const int t = min(i, E.n - 1) / ld, l = i % ld;
         const int2 s = ul.off[t * ul.KY], e = ul.off[(t + 1) * ul.KY];
         if (s.x >= e.x) return;
         const int tot = ul.off[ul.TT * ul.KY].y;
         const int b0 = ul.block_of(s.y, tot), b1 = ul.block_of(ul.list[e.x - 1].y, tot), rows = E.comp ? 2 * ncomp : ncomp;
-        for (int b = b0 + part_i; b <= b1; b += PARTS) add(part + (size_t)(b + t) * rows * ld + l, ncomp, ld);
+        for (int b = b0 + part_i; b <= b1; b += PARTS) add(part + (size_t)(b + t) * rows * ld + l, ncomp, ldc);
     };
     if (E.far) {
-        add_list(E.ulf, E.part_f, E.ncomp_f, TGT_TILE);
+        add_list(E.ulf, E.part_f, E.ncomp_f, Whole{});
         if (E.ncomp == 17) {
             // the far units' transposed stretching (times 4 pi) from their sums, Gamma_i x S - 3 G'^T Gamma_i
             const float4 g = reinterpret_cast<const float4*>(E.o.str)[min(i, E.n - 1)];
@@ -624,25 +650,32 @@ __global__ void __launch_bounds__(256) epilogue_kernel(const EpiArgs E)
 #pragma unroll
             for (int c = 0; c < 3; ++c) H[14 + c] = (float)s[c], Lw[14 + c] = (float)(s[c] - (double)H[14 + c]);
         }
-        add_list(E.uln, E.part, E.ncomp, FAR_GROUP);
+        add_list(E.uln, E.part, E.ncomp, Team{});
     }
-    // the partial sums of the particle launch, then those of the segment launch
-    for (int launch = E.far ? 1 : 0; launch < 2; ++launch) {
-        const StreamK& sk = launch ? E.sks : E.sk;
-        const float* part = launch ? E.part_s : E.part;
+    auto add_stream = [&](const StreamK& sk, const float* part, auto ldc) {
+        constexpr int ld = decltype(ldc)::value;
         const int nunits = sk.np + sk.ns;
-        if (nunits == 0) continue;
+        if (nunits == 0) return;
+        const int t = min(i, E.n - 1) / ld, l = i % ld, rows = E.comp ? 2 * E.ncomp : E.ncomp;
         const int b0 = sk.block_of(sk.unit_start(t, 0));
         const int b1 = sk.block_of(sk.unit_start(t, nunits - 1));
-        const int rows = E.comp ? 2 * E.ncomp : E.ncomp;
         for (int b = b0 + part_i; b <= b1; b += PARTS) {
             const long long lo_b = sk.lo(b), hi_b = sk.lo(b + 1);
             long long c0 = lo_b > (long long)t * sk.C ? lo_b : (long long)t * sk.C;
             int tt, kk;
             sk.first_at_or_after(c0, tt, kk);
             if (tt != t || sk.unit_start(tt, kk) >= hi_b) continue;  // block b ran no unit of tile t
-            add(part + (size_t)(b + t) * rows * TGT_TILE + l, E.ncomp, TGT_TILE);
+            add(part + (size_t)(b + t) * rows * ld + l, E.ncomp, ldc);
         }
+    };
+    // the partial sums of the particle launch, then those of the segment launch
+    for (int launch = E.far ? 1 : 0; launch < 2; ++launch) {
+        const StreamK& sk = launch ? E.sks : E.sk;
+        const float* part = launch ? E.part_s : E.part;
+        if ((launch ? E.tgt_s : E.tgt) == TGT_TILE)
+            add_stream(sk, part, Whole{});
+        else
+            add_stream(sk, part, Team{});
     }
     if constexpr (PARTS > 1) {  // fold the parts, in order
         __shared__ float sh[17][2][256];
@@ -737,14 +770,14 @@ __global__ void __launch_bounds__(256) epilogue_kernel(const EpiArgs E)
 // Each block owns 64 consecutive particles (two per lane of every warp) with two bounding
 // boxes (split at the largest index-order jump).  Its warps walk the source tiles 32 at a
 // time, one box test per lane, and share the tiles within 7 sigma of either box among
-// them, tile by tile: a warp stages its tile (positions, strengths, nu_t) in its own slice
-// of shared memory with coalesced loads, then every lane sums over it; the warps' sums are
-// added in a fixed order.  (One warp per 64 particles left most SMs idle below 50,000
-// particles: 71 us for 2,000 and 86 us for 20,000, 30 and 33 us so.)  v_i Gamma_j - v_j Gamma_i is formed from two
+// them, 32 sources at a time: a warp stages its sources (positions, strengths, nu_t) in its
+// own slice of shared memory with coalesced loads, then every lane sums over them; the
+// warps' sums are added in a fixed order.  (One warp per 64 particles left most SMs idle
+// below 50,000 particles: 71 us for 2,000 and 86 us for 20,000; eight warps 30 and 33 us.)  v_i Gamma_j - v_j Gamma_i is formed from two
 // rounded products so that the i == j term is exactly zero; pairs beyond 7 sigma
 // get exp(-r^2/2s^2) < 3e-11 and are skipped.
 // ---------------------------------------------------------------------------
-constexpr int PSE_T = 256;
+constexpr int PSE_T = 512;
 constexpr int PSE_W = PSE_T / 32;
 
 __device__ __forceinline__ void pse_pair(float4 pi, float4 gi, float base, float4 pj, float4 gj, float ntj,
@@ -767,8 +800,8 @@ __global__ void __launch_bounds__(PSE_T) pse_kernel(const float4* __restrict__ p
                                                     float cut2, float nu, float pref, const int* __restrict__ perm,
                                                     float* __restrict__ dGdt)
 {
-    __shared__ float4 sp[PSE_W][SRC_TILE], sg[PSE_W][SRC_TILE];
-    __shared__ float snt[PSE_W][SRC_TILE];
+    __shared__ float4 stage[2][PSE_W][32];  // positions and strengths; the warps' sums at the end
+    __shared__ float snt[PSE_W][32];
     __shared__ float wbox[PSE_W][12];
     __shared__ unsigned found[2][PSE_W];  // tiles in reach, 32 per warp: this round's and the last one's
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -781,7 +814,11 @@ __global__ void __launch_bounds__(PSE_T) pse_kernel(const float4* __restrict__ p
     warp_two_boxes(make_float3(p0.x, p0.y, p0.z), v0, make_float3(p1.x, p1.y, p1.z), v1, wbox[warp]);
     const float base0 = nu + 0.5f * nt0, base1 = nu + 0.5f * nt1;
     float a0x = 0.f, a0y = 0.f, a0z = 0.f, a1x = 0.f, a1y = 0.f, a1z = 0.f;
-    int met = 0;  // tiles in reach so far: warp w takes those with number = w (mod PSE_W)
+    float4* sp = stage[0][warp];
+    float4* sg = stage[1][warp];
+    // warp w takes the 32 sources w mod 4 of the tiles in reach whose number is w / 4 (mod PSE_W / 4)
+    const int word = warp & 3, slot = warp >> 2;
+    int met = 0;  // tiles in reach so far
     for (int tb = 0, r = 0; tb < ntiles; tb += 32 * PSE_W, r ^= 1) {
         const int tt = tb + 32 * warp + lane;
         const bool near = tt < ntiles && boxes_near(wbox[warp], box[2 * tt], box[2 * tt + 1], cut2);
@@ -791,34 +828,26 @@ __global__ void __launch_bounds__(PSE_T) pse_kernel(const float4* __restrict__ p
 #pragma unroll 1
         for (int w = 0; w < PSE_W; ++w)
         for (unsigned mask = found[r][w]; mask; mask &= mask - 1, ++met) {
-            if ((met & (PSE_W - 1)) != warp) continue;
-            const int tile = tb + 32 * w + __ffs(mask) - 1;
-            const int j0 = tile * SRC_TILE, cnt = min(SRC_TILE, n - j0);
-            __syncwarp();
-            // stage the tile; a source at least 7 sigma from both of the warp's target boxes
+            if ((met & (PSE_W / 4 - 1)) != slot) continue;
+            const int j = (tb + 32 * w + __ffs(mask) - 1) * SRC_TILE + 32 * word + lane;
+            // stage the sources; one at least 7 sigma from both of the warp's target boxes
             // reaches none of its targets and is left out (warp-uniformly, by ballot)
-            unsigned keep[SRC_TILE / 32];
-#pragma unroll
-            for (int h = 0; h < SRC_TILE / 32; ++h) {
-                const int q = lane + 32 * h;
-                bool kp = false;
-                if (q < cnt) {
-                    const float4 pq = pos[j0 + q];
-                    sp[warp][q] = pq;
-                    sg[warp][q] = str[j0 + q];
-                    snt[warp][q] = nu_t ? nu_t[j0 + q] : 0.f;
-                    const float4 pt = make_float4(pq.x, pq.y, pq.z, 0.f);
-                    kp = boxes_near(wbox[warp], pt, pt, cut2);
-                }
-                keep[h] = __ballot_sync(0xffffffffu, kp);
-            }
             __syncwarp();
-#pragma unroll
-            for (int h = 0; h < SRC_TILE / 32; ++h)
-            for (unsigned m = keep[h]; m; m &= m - 1) {
-                const int j = 32 * h + __ffs(m) - 1;
-                const float4 pj = sp[warp][j], gj = sg[warp][j];
-                const float ntj = snt[warp][j];
+            bool kp = false;
+            if (j < n) {
+                const float4 pq = pos[j];
+                sp[lane] = pq;
+                sg[lane] = str[j];
+                snt[warp][lane] = nu_t ? nu_t[j] : 0.f;
+                const float4 pt = make_float4(pq.x, pq.y, pq.z, 0.f);
+                kp = boxes_near(wbox[warp], pt, pt, cut2);
+            }
+            unsigned m = __ballot_sync(0xffffffffu, kp);
+            __syncwarp();
+            for (; m; m &= m - 1) {
+                const int q = __ffs(m) - 1;
+                const float4 pj = sp[q], gj = sg[q];
+                const float ntj = snt[warp][q];
                 pse_pair(p0, g0, base0, pj, gj, ntj, inv2s2, cut2, a0x, a0y, a0z);
                 pse_pair(p1, g1, base1, pj, gj, ntj, inv2s2, cut2, a1x, a1y, a1z);
             }
@@ -826,7 +855,7 @@ __global__ void __launch_bounds__(PSE_T) pse_kernel(const float4* __restrict__ p
     }
     // the warps' sums in a fixed order, one thread per target
     __syncthreads();
-    float4* sums = &sp[0][0];  // [PSE_W][64]
+    float4* sums = &stage[0][0][0];  // [PSE_W][64]
     sums[warp * 64 + lane] = make_float4(a0x, a0y, a0z, 0.f);
     sums[warp * 64 + 32 + lane] = make_float4(a1x, a1y, a1z, 0.f);
     __syncthreads();
@@ -947,7 +976,9 @@ static int blocks_per_sm_kind(bool g, bool c, bool s)
 static int blocks_per_sm(bool g, bool c, bool s, int kind)
 {
     return kind == SWEEP_SEGMENTS ? blocks_per_sm_kind<SWEEP_SEGMENTS>(g, c, s)
+           : kind == SWEEP_SEG_SMALL ? blocks_per_sm_kind<SWEEP_SEG_SMALL>(g, c, s)
            : kind == SWEEP_NEAR   ? blocks_per_sm_kind<SWEEP_NEAR>(g, c, s)
+           : kind == SWEEP_SMALL  ? blocks_per_sm_kind<SWEEP_SMALL>(g, c, s)
                                   : blocks_per_sm_kind<SWEEP_PARTICLES>(g, c, s);
 }
 
@@ -971,39 +1002,45 @@ SweepPlan plan_sweep(int64_t n_tgt, int64_t n_src, int64_t m_seg, bool grad, boo
     p.TT = (int)((n_tgt + TGT_TILE - 1) / TGT_TILE);
     p.SP = (int)((n_src + SRC_TILE - 1) / SRC_TILE);
     p.SS = (int)((m_seg + SRC_TILE - 1) / SRC_TILE);
+    const long long units_p = (long long)p.TT * p.SP;
+    const bool far_size =
+        allow_far && (units_p >= FAR_MIN_UNITS || (n_tgt == n_src && grad && n_src >= FAR_SORT_MIN));
+    p.far = far_size && units_p <= FAR_MAX_UNITS;
     // particle tiles and segment tiles: one stream-K plan (and launch) each
-    auto plan = [&](StreamK& sk, int np, int ns) {
-        sk.TT = p.TT;
-        sk.np = np;
-        sk.ns = ns;
+    auto plan = [&](StreamK& sk, int kind, int np, int ns) {
+        const bool teams = kind == SWEEP_SMALL || kind == SWEEP_SEG_SMALL;
+        const int per_tile = teams ? Ring<SWEEP_SMALL>::PER_TILE : 1;
+        const int tgt = teams ? Ring<SWEEP_SMALL>::TGT : TGT_TILE;
+        sk.TT = (int)((n_tgt + tgt - 1) / tgt);
+        sk.np = np * per_tile;
+        sk.ns = ns * per_tile;
         sk.wp = UNIT_W_P;
         sk.ws = grad ? UNIT_W_S_GRAD : UNIT_W_S_VEL;
         sk.C = (long long)sk.np * sk.wp + (long long)sk.ns * sk.ws;
         sk.tot = (long long)sk.TT * sk.C;
         const long long units = (long long)sk.TT * (sk.np + sk.ns);
-        long long B = sweep_blocks(grad, comp, p.stretch, ns > 0 ? SWEEP_SEGMENTS : SWEEP_PARTICLES);
+        long long B = (long long)sweep_blocks(grad, comp, p.stretch, kind) * (teams ? Ring<SWEEP_SMALL>::TEAMS : 1);
         if (B > units) B = units;
         if (B < 1) B = 1;
         sk.B = (int)B;
     };
-    // A small problem (fewer cost units than four waves of resident blocks) sweeps both
-    // kinds of tile in one launch; a larger one gives the segment tiles a launch of
-    // their own, where closed rings are packed by corner.
-    const long long units_all = (long long)p.TT * (p.SP + p.SS);
-    p.mixed = p.SP > 0 && p.SS > 0 && units_all < 4LL * sweep_blocks(grad, comp, p.stretch);
-    plan(p.sk, p.SP, p.mixed ? p.SS : 0);
-    plan(p.sks, 0, p.mixed ? 0 : p.SS);
+    // A small problem with few segments sweeps both kinds of tile in one launch; otherwise the
+    // segment tiles have a launch of their own, where closed rings are packed by corner.
+    const long long units_s = (long long)p.TT * p.SS;
+    p.mixed = p.SP > 0 && p.SS > 0 && p.SS <= MIXED_MAX_TILES && !p.far && units_p < SMALL_MAX_UNITS;
+    p.kind = units_p < SMALL_MAX_UNITS ? SWEEP_SMALL : SWEEP_PARTICLES;
+    p.kind_s = units_s < SEG_SMALL_MAX_UNITS ? SWEEP_SEG_SMALL : SWEEP_SEGMENTS;
+    plan(p.sk, p.kind, p.SP, p.mixed ? p.SS : 0);
+    plan(p.sks, p.kind_s, 0, p.mixed ? 0 : p.SS);
+    const size_t tgt_k = p.kind == SWEEP_SMALL ? Ring<SWEEP_SMALL>::TGT : TGT_TILE,
+                 tgt_s = p.kind_s == SWEEP_SEG_SMALL ? Ring<SWEEP_SEG_SMALL>::TGT : TGT_TILE;
     p.off_psrc = cv.take((size_t)p.SP * SRC_TILE * P_F4 * 16);
     p.off_pbox = cv.take((size_t)p.SP * 2 * 16);
     p.off_ssrc = cv.take((size_t)p.SS * SRC_TILE * S_F4 * 16);
     p.off_sbox = cv.take((size_t)p.SS * 2 * 16);
     const size_t rows = (size_t)(comp ? 2 : 1) * p.ncomp;
-    const long long units_p = (long long)p.TT * p.SP;
-    const bool far_size =
-        allow_far && (units_p >= FAR_MIN_UNITS || (n_tgt == n_src && grad && n_src >= FAR_SORT_MIN));
-    p.far = far_size && units_p <= FAR_MAX_UNITS;
-    if (!p.far && p.sk.np + p.sk.ns > 0) p.off_part = cv.take((size_t)(p.sk.TT + p.sk.B) * rows * TGT_TILE * sizeof(float));
-    if (p.sks.ns > 0) p.off_part_s = cv.take((size_t)(p.sks.TT + p.sks.B) * rows * TGT_TILE * sizeof(float));
+    if (!p.far && p.sk.np + p.sk.ns > 0) p.off_part = cv.take((size_t)(p.sk.TT + p.sk.B) * rows * tgt_k * sizeof(float));
+    if (p.sks.ns > 0) p.off_part_s = cv.take((size_t)(p.sks.TT + p.sks.B) * rows * tgt_s * sizeof(float));
     // Units on the tensor cores
     if (far_size) {
         p.KY = (p.SP + FAR_KCH - 1) / FAR_KCH;
@@ -1037,8 +1074,12 @@ SweepPlan plan_sweep(int64_t n_tgt, int64_t n_src, int64_t m_seg, bool grad, boo
 template <bool G, bool C, bool S>
 static void launch_sweep(const SweepArgs& A, int B, int kind, cudaStream_t st)
 {
-    if (kind == SWEEP_NEAR)
+    if (kind == SWEEP_SEG_SMALL)
+        sweep_kernel<G, C, S, SWEEP_SEG_SMALL><<<B, SWEEP_TPB, sweep_smem_bytes<G, C, S, SWEEP_SEG_SMALL>(), st>>>(A);
+    else if (kind == SWEEP_NEAR)
         sweep_kernel<G, C, S, SWEEP_NEAR><<<B, SWEEP_TPB, sweep_smem_bytes<G, C, S, SWEEP_NEAR>(), st>>>(A);
+    else if (kind == SWEEP_SMALL)
+        sweep_kernel<G, C, S, SWEEP_SMALL><<<B, SWEEP_TPB, sweep_smem_bytes<G, C, S, SWEEP_SMALL>(), st>>>(A);
     else if (kind == SWEEP_SEGMENTS)
         sweep_kernel<G, C, S, SWEEP_SEGMENTS><<<B, SWEEP_TPB, sweep_smem_bytes<G, C, S, SWEEP_SEGMENTS>(), st>>>(A);
     else
@@ -1100,7 +1141,7 @@ cudaError_t run_sweep(const SweepPlan& p, char* ws, const float* tgt, const floa
         };
         uln = list(p.off_nlist, p.off_noff, p.TT * FAR_GROUPS, p.B_near * Ring<SWEEP_NEAR>::TEAMS,
                    Ring<SWEEP_NEAR>::WARPS * NEAR_COST);
-        ulf = list(p.off_flist, p.off_foff, p.TT, p.B_far, FAR_GROUPS);
+        ulf = list(p.off_flist, p.off_foff, p.TT, p.B_far, FAR_COST_FIRST + FAR_GROUPS - 1);
         cudaError_t e = run_far_pack(reinterpret_cast<const float4*>(src_pos), reinterpret_cast<const float4*>(src_str),
                                      p.n_src, pbox, p.SP, p.grad, reinterpret_cast<unsigned char*>(ws + p.off_ftile), st);
         if (e == cudaSuccess)
@@ -1114,8 +1155,8 @@ cudaError_t run_sweep(const SweepPlan& p, char* ws, const float* tgt, const floa
     }
     if (p.SP + p.SS > 0) {
         // shared-memory opt-in
-        if (p.sk.np + p.sk.ns > 0) blocks_per_sm(p.grad, p.comp, p.stretch, p.far ? SWEEP_NEAR : SWEEP_PARTICLES);
-        if (p.sks.ns > 0) blocks_per_sm(p.grad, p.comp, p.stretch, SWEEP_SEGMENTS);
+        if (p.sk.np + p.sk.ns > 0) blocks_per_sm(p.grad, p.comp, p.stretch, p.far ? SWEEP_NEAR : p.kind);
+        if (p.sks.ns > 0) blocks_per_sm(p.grad, p.comp, p.stretch, p.kind_s);
         SweepArgs A;
         A.tgt = reinterpret_cast<const float4*>(tgt);
         A.tstr = p.stretch ? reinterpret_cast<const float4*>(own) : nullptr;
@@ -1141,8 +1182,11 @@ cudaError_t run_sweep(const SweepPlan& p, char* ws, const float* tgt, const floa
             TraceScope ts(seg ? VPM_TRACE_SEGMENTS : p.grad ? VPM_TRACE_SWEEP : VPM_TRACE_SWEEP_VEL, st);
             A.sk = seg ? p.sks : p.sk;
             A.part = seg ? part_s : part;
-            const int B = !seg && p.far ? p.B_near : A.sk.B;
-            const int k = seg ? SWEEP_SEGMENTS : p.far ? SWEEP_NEAR : SWEEP_PARTICLES;
+            const int k = seg ? p.kind_s : p.far ? SWEEP_NEAR : p.kind;
+            // with teams: a block for each of the first teams, up to the resident number
+            const int B = k == SWEEP_NEAR    ? p.B_near
+                          : k == SWEEP_PARTICLES || k == SWEEP_SEGMENTS ? A.sk.B
+                                             : std::min(A.sk.B, sweep_blocks(p.grad, p.comp, p.stretch, k));
             if (k == SWEEP_NEAR) {
                 A.ul = uln;
                 A.part = reinterpret_cast<float*>(ws + p.off_part_n);
@@ -1180,6 +1224,8 @@ cudaError_t run_sweep(const SweepPlan& p, char* ws, const float* tgt, const floa
     E.part = p.far ? reinterpret_cast<const float*>(ws + p.off_part_n) : part;
     E.sks = p.sks;
     E.part_s = part_s;
+    E.tgt = p.kind == SWEEP_SMALL ? Ring<SWEEP_SMALL>::TGT : TGT_TILE;
+    E.tgt_s = p.kind_s == SWEEP_SEG_SMALL ? Ring<SWEEP_SEG_SMALL>::TGT : TGT_TILE;
     E.far = p.far ? 1 : 0;
     E.uln = uln;
     E.ulf = ulf;
@@ -1195,7 +1241,9 @@ cudaError_t run_sweep(const SweepPlan& p, char* ws, const float* tgt, const floa
     trace_launch();
     // Threads per target: enough to give every SM a few blocks
     const long long want = 4LL * 256 * std::max(sm_count(), 1);
-    if (2LL * p.n_tgt <= want)
+    if (16LL * p.n_tgt <= want)
+        epilogue_kernel<16><<<(p.n_tgt + 15) / 16, 256, 0, st>>>(E);
+    else if (2LL * p.n_tgt <= want)
         epilogue_kernel<8><<<(p.n_tgt + 31) / 32, 256, 0, st>>>(E);
     else
         epilogue_kernel<1><<<(p.n_tgt + 255) / 256, 256, 0, st>>>(E);
