@@ -52,10 +52,11 @@ constexpr int FAR_COST_FIRST = 3;                // cost of a far unit's first g
 // (hover wake, 100,000: 7.20 ms at 0.2, 6.23 at 0.33, 5.88 at 0.5, 5.63 at 0.6).
 constexpr float FAR_TAU = 0.5f;
 // (1,024-target, 128-source) units from which the far sweep is used: below, packing and
-// listing (about 40 us) cost more than it saves.  1,280 control points, velocity only:
+// listing (about 40 us) cost more than it saves.  Velocity only, 1,280 control points:
 // 100,000 sources (1,564 units) 176 us without it and 185 us with it, 150,000 (2,344 units)
-// 240 and 229 us.
-constexpr long long FAR_MIN_UNITS = 2048;
+// 240 and 229 us.  With the gradient, the adjoint of 1,280 control points at 60,000 particles
+// (590 units) 185 and 235 us, at 110,000 (1,080 units) 223 and 196 us.
+constexpr long long FAR_MIN_UNITS_VEL = 2048, FAR_MIN_UNITS_GRAD = 900;
 constexpr long long FAR_MAX_UNITS = 1LL << 26;   // ... and to which (the unit lists take up to 44 bytes each)
 // Particles onto themselves: smallest count put in curve order and swept this way (right-hand
 // side of the BVI wake: 16,000 particles 819 us without and 744 us with it, 12,000 particles

@@ -78,7 +78,7 @@ SweepPlan plan_sweep(int64_t n_tgt, int64_t n_src, int64_t m_seg, bool grad, boo
 
 // Launches packing, the sweep and the reduction/epilogue.
 struct EpilogueOut {
-    int mode = 0;  // 0: velocity (+gradient) outputs; 1: right-hand side
+    int mode = 0;  // 0: velocity (+gradient) outputs; 1: right-hand side; 2: adjoint (u to dGdt, J^T Gamma to dxdt)
     float* u = nullptr;
     float* grad_u = nullptr;
     const float* str = nullptr;  // particle strengths (rhs)

@@ -728,6 +728,13 @@ __global__ void __launch_bounds__(256) epilogue_kernel(const EpiArgs E)
         }
         return;
     }
+    if (o.mode == 2) {  // the adjoint at particle i
+        o.dGdt[d] = (float)u0;
+        o.dGdt[E.n + d] = (float)u1;
+        o.dGdt[2 * E.n + d] = (float)u2;
+        for (int a = 0; a < 3; ++a) o.dxdt[(size_t)a * E.n + d] = (float)(acc[14 + a] * f4pi);
+        return;
+    }
     // Right-hand side of Eq. 4-5 for particle i.
     const float4 G4 = reinterpret_cast<const float4*>(o.str)[i];
     const double Gm[3] = {G4.x, G4.y, G4.z};
@@ -1004,7 +1011,8 @@ SweepPlan plan_sweep(int64_t n_tgt, int64_t n_src, int64_t m_seg, bool grad, boo
     p.SS = (int)((m_seg + SRC_TILE - 1) / SRC_TILE);
     const long long units_p = (long long)p.TT * p.SP;
     const bool far_size =
-        allow_far && (units_p >= FAR_MIN_UNITS || (n_tgt == n_src && grad && n_src >= FAR_SORT_MIN));
+        allow_far && (n_tgt == n_src && grad ? n_src >= FAR_SORT_MIN
+                                             : units_p >= (grad ? FAR_MIN_UNITS_GRAD : FAR_MIN_UNITS_VEL));
     p.far = far_size && units_p <= FAR_MAX_UNITS;
     // particle tiles and segment tiles: one stream-K plan (and launch) each
     auto plan = [&](StreamK& sk, int kind, int np, int ns) {
@@ -1179,7 +1187,7 @@ cudaError_t run_sweep(const SweepPlan& p, char* ws, const float* tgt, const floa
         for (int kind = 0; kind < 2; ++kind) {
             const bool seg = kind == 1;
             if ((seg ? p.sks.ns : p.sk.np + p.sk.ns) == 0) continue;
-            TraceScope ts(seg ? VPM_TRACE_SEGMENTS : p.grad ? VPM_TRACE_SWEEP : VPM_TRACE_SWEEP_VEL, st);
+            TraceScope ts(seg ? VPM_TRACE_SEGMENTS : out.mode == 2 ? VPM_TRACE_ADJOINT : p.grad ? VPM_TRACE_SWEEP : VPM_TRACE_SWEEP_VEL, st);
             A.sk = seg ? p.sks : p.sk;
             A.part = seg ? part_s : part;
             const int k = seg ? p.kind_s : p.far ? SWEEP_NEAR : p.kind;

@@ -114,3 +114,23 @@ def test_stretching_of_far_units(api):
         ref = oracle.stretch(J + Js, w.strength[idx], classic)
         assert rel_l2(dx[:, idx].double().cpu().numpy().T, u + us) <= TOL_COMP
         assert rel_l2(dG[:, idx].double().cpu().numpy().T, ref) <= TOL_COMP
+
+
+@pytest.mark.parametrize("n,k", [(115_300, 1000), (30_721, 4000), (930_000, 1), (460_801, 129)])
+@pytest.mark.parametrize("compensated", [True, False])
+def test_adjoint_by_the_sweep(api, n, k, compensated):
+    """The adjoint of a problem large enough for the tensor cores: the particle sweep with the points as sources."""
+    w = synth.multirotor(seed=9, n=n)
+    rng = np.random.default_rng(4)
+    pts = _pad(rng.uniform([-2, -1, -0.6], [2, 1, 0.3], size=(k, 3)))
+    pts[0, :3] = w.pos[n // 2, :3]  # a point on a particle: nothing from that pair
+    g = _f32(rng.normal(size=(3, k)))
+    dx, dG = api.induce_backward(to_dev(w.pos), to_dev(w.strength), to_dev(pts), w.sigma, to_dev(g),
+                                 compensated=compensated)
+    torch.cuda.synchronize()
+    assert api.device_error() == 0
+    idx = np.unique(np.concatenate([[0, n // 2, n - 1], synth.sample_targets(6, n, 3000)]))
+    rx, rG = oracle.p2p_adjoint(w.pos[idx], w.strength[idx], pts, w.sigma, g.T)
+    tol = 1e-5 if compensated else 1e-3
+    assert rel_l2(dx[:, idx].double().cpu().numpy().T, rx) <= tol
+    assert rel_l2(dG[:, idx].double().cpu().numpy().T, rG) <= tol
