@@ -13,6 +13,7 @@
 #include <math.h>
 
 #include <algorithm>
+#include <type_traits>
 
 #include <cooperative_groups.h>
 
@@ -952,6 +953,318 @@ __global__ void __launch_bounds__(256) residual_kernel(const float* __restrict__
     if (blockIdx.x == 0 && threadIdx.x == 0) out[4] = (double)info[0], out[5] = (double)info[1];
 }
 
+// ---------------------------------------------------------------------------
+// Small row-dominant systems in one block: the whole solve (dominance test, LU without row
+// exchanges, substitutions, FP64 residuals and corrections) with the matrix in shared
+// memory.  The chain of launches of the general path costs 7 to 12 us a step whatever the
+// order, and each refinement a host synchronisation; here it is one launch and one
+// synchronisation (order 160, build and solve: 220 -> 172 us).  Bound by serial chains: at
+// order 160 the panels take half of the kernel's time (a column about 0.4 us: the pivot row
+// through shared memory, a barrier, the reciprocal), the two FP64 residuals a quarter.
+// out: 0 converged, 1 not converged (best iterate in x), 2 not row-dominant or no usable
+// pivot (nothing in x); corrections made; backward error.
+// ---------------------------------------------------------------------------
+constexpr int SMALL_N = 224, SMALL_T = 512, SMALL_W = SMALL_T / 32;
+constexpr int SMALL_PT = 256;  // threads of a panel
+static_assert(SMALL_PT >= SMALL_N, "a thread per row");
+
+__host__ __device__ constexpr int small_ld(int n) { return n | 1; }  // odd: columns without bank conflicts
+__host__ __device__ constexpr size_t small_smem(int n)
+{
+    return (size_t)n * 4 * sizeof(double) + ((size_t)n * small_ld(n) + n + 32) * sizeof(float);
+}
+
+// 1 / d to within an ulp, in a few instructions.
+__device__ __forceinline__ float small_rcp(float d)
+{
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(d));
+    return fmaf(fmaf(-d, r, 1.f), r, r);
+}
+
+__global__ void __launch_bounds__(SMALL_T, 1) aic_small_kernel(const float* __restrict__ A,
+                                                               const double* __restrict__ b, double* __restrict__ x,
+                                                               int n, double tol, int max_iter,
+                                                               double* __restrict__ out)
+{
+    extern __shared__ __align__(16) double dsm[];
+    __shared__ __align__(16) float prow[2][NB + 4];  // the pivot rows of this step and the next, and their pivots' reciprocals
+    __shared__ unsigned long long nrm[4];  // bits of the largest |r|, |x|, row sum, |b|; non-negative doubles order as integers
+    double* xs = dsm;
+    double* rs = xs + n;
+    double* xb = rs + n;
+    double* ra = xb + n;  // row sums of |a|
+    float* LU = reinterpret_cast<float*>(ra + n);
+    const int ld = small_ld(n), tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    float* y = LU + (size_t)n * ld;  // n + 32
+
+    for (int c = lane; c < n; c += 32)
+#pragma unroll 8
+        for (int i = warp; i < n; i += SMALL_W) LU[i * ld + c] = A[(size_t)i * n + c];
+    __syncthreads();
+    // two threads per row (2 n <= SMALL_T) for the sums over rows
+    const int ri = tid >> 1, rh = tid & 1;
+    bool bad = false;
+    {
+        float s = 0.f, e = 0.f;  // sum of |a| in double-float (48 bits)
+        if (ri < n)
+            for (int c = rh; c < n; c += 2) {
+                float t;
+                two_sum(s, fabsf(LU[ri * ld + c]), s, t);
+                e += t;
+            }
+        float t;
+        const float so = __shfl_xor_sync(0xffffffffu, s, 1);
+        two_sum(fmaxf(s, so), fminf(s, so), s, t);
+        e += __shfl_xor_sync(0xffffffffu, e, 1) + t;
+        if (ri < n) {
+            const double sum = (double)s + (double)e;
+            if (rh == 0) ra[ri] = sum;
+            bad = !(2.0 * fabs((double)LU[ri * ld + ri]) > sum);
+        }
+    }
+    if (__syncthreads_or(bad)) {
+        if (tid == 0) out[0] = 2.0;
+        return;
+    }
+    for (int k0 = 0; k0 < n; k0 += NB) {
+        const int nb = min(NB, n - k0), c0 = k0 + nb, rest = n - c0;
+        // The panel: a row per thread, its entries in registers; at step j the pivot row (and
+        // its pivot's reciprocal) comes through shared memory.
+        bool zero = false;
+        if (tid < SMALL_PT) {
+            const int i = k0 + tid;
+            float v[NB];
+#pragma unroll
+            for (int c = 0; c < NB; ++c) v[c] = i < n && c < nb ? LU[i * ld + k0 + c] : (c == tid ? 1.f : 0.f);
+            auto send = [&](int j) {  // by the thread of row j
+#pragma unroll
+                for (int c = 0; c < NB; c += 4)
+                    *reinterpret_cast<float4*>(&prow[j & 1][c]) = make_float4(v[c], v[c + 1], v[c + 2], v[c + 3]);
+                float d = v[0];
+#pragma unroll
+                for (int c = 1; c < NB; ++c)
+                    if (c == j) d = v[c];
+                prow[j & 1][NB] = small_rcp(d);
+            };
+            if (tid == 0) send(0);
+#pragma unroll
+            for (int j = 0; j < NB; ++j) {
+                __syncwarp();  // the rows' branches below leave warp 0 diverged
+                asm volatile("barrier.cta.sync 1, %0;" ::"n"(SMALL_PT) : "memory");
+                const float rj = prow[j & 1][NB];
+                zero = zero || !(fabsf(rj) > 0.f) || !isfinite(rj);  // a zero, infinite or NaN pivot
+                if (tid > j) {
+                    const float l = v[j] * rj;
+                    v[j] = l;
+#pragma unroll
+                    for (int c = j + 1; c < NB; ++c) v[c] = fmaf(-l, prow[j & 1][c], v[c]);
+                    if (j + 1 < NB && tid == j + 1) send(j + 1);
+                }
+            }
+#pragma unroll
+            for (int c = 0; c < NB; ++c)
+                if (i < n && c < nb) LU[i * ld + k0 + c] = v[c];
+        }
+        if (__syncthreads_or(zero)) {
+            if (tid == 0) out[0] = 2.0;
+            return;
+        }
+        if (rest <= 0) break;  // (with rest > 0 the panel is NB wide)
+        if (tid < rest) {  // U12 = L11^-1 A12: a column per thread
+            float* col = LU + k0 * ld + c0 + tid;
+            float v[NB];
+#pragma unroll
+            for (int i = 0; i < NB; ++i) {
+                float e[4] = {col[i * ld], 0.f, 0.f, 0.f};
+#pragma unroll
+                for (int p = 0; p < i; ++p) e[p & 3] = fmaf(-LU[(k0 + i) * ld + k0 + p], v[p], e[p & 3]);
+                v[i] = (e[0] + e[1]) + (e[2] + e[3]);
+            }
+#pragma unroll
+            for (int i = 1; i < NB; ++i) col[i * ld] = v[i];
+        }
+        __syncthreads();
+        // A22 -= L21 U12: four rows a warp at a time, NC columns a lane (loads beyond the
+        // matrix are clamped into it, their results dropped)
+        auto update = [&](auto nc) {
+            constexpr int NC = decltype(nc)::value;
+            int col[NC];
+#pragma unroll
+            for (int r = 0; r < NC; ++r) col[r] = min(c0 + lane + 32 * r, n - 1);
+#pragma unroll 1
+            for (int i0 = c0 + 4 * warp; i0 < n; i0 += 4 * SMALL_W) {
+                float acc[4][NC];
+                const float* row[4];
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    row[q] = LU + min(i0 + q, n - 1) * ld;
+#pragma unroll
+                    for (int r = 0; r < NC; ++r) acc[q][r] = 0.f;  // one rounding against the entry, not 32
+                }
+#pragma unroll 4
+                for (int p = k0; p < c0; ++p) {
+                    float u[NC];
+#pragma unroll
+                    for (int r = 0; r < NC; ++r) u[r] = LU[p * ld + col[r]];
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) {
+                        const float l = row[q][p];
+#pragma unroll
+                        for (int r = 0; r < NC; ++r) acc[q][r] = fmaf(l, u[r], acc[q][r]);
+                    }
+                }
+#pragma unroll
+                for (int q = 0; q < 4; ++q)
+#pragma unroll
+                    for (int r = 0; r < NC; ++r)
+                        if (i0 + q < n && c0 + lane + 32 * r < n) LU[(i0 + q) * ld + c0 + lane + 32 * r] -= acc[q][r];
+            }
+        };
+        switch ((rest + 31) / 32) {
+            case 1: update(std::integral_constant<int, 1>{}); break;
+            case 2: update(std::integral_constant<int, 2>{}); break;
+            case 3: update(std::integral_constant<int, 3>{}); break;
+            case 4: update(std::integral_constant<int, 4>{}); break;
+            case 5: update(std::integral_constant<int, 5>{}); break;
+            default: update(std::integral_constant<int, 6>{}); break;
+        }
+        __syncthreads();
+    }
+    // The diagonal blocks are replaced by the inverses of their factors (unit lower and upper
+    // triangle in place), a warp each (2 nblk <= SMALL_W): lane = column.
+    {
+        static_assert(2 * ((SMALL_N + NB - 1) / NB) <= SMALL_W, "a warp per triangle");
+        const int nblk = (n + NB - 1) / NB;
+        const bool low = warp < nblk, mine = warp < 2 * nblk;
+        const int k0 = NB * (low ? warp : warp - nblk), nb = min(NB, n - k0);
+        float v[NB];
+        if (mine) {
+            const float* D = LU + k0 * ld + k0;
+            if (low) {
+#pragma unroll
+                for (int i = 0; i < NB; ++i) {
+                    float e[2] = {i == lane ? 1.f : 0.f, 0.f};
+                    if (i < nb)
+#pragma unroll
+                        for (int p = 0; p < i; ++p) e[p & 1] = fmaf(-D[i * ld + p], v[p], e[p & 1]);
+                    v[i] = e[0] + e[1];
+                }
+            } else {
+#pragma unroll
+                for (int i = NB - 1; i >= 0; --i) {
+                    float e[2] = {i == lane ? 1.f : 0.f, 0.f}, r = 1.f;
+                    if (i < nb) {
+                        r = small_rcp(D[i * ld + i]);
+#pragma unroll
+                        for (int p = i + 1; p < NB; ++p)
+                            if (p < nb) e[p & 1] = fmaf(-D[i * ld + p], v[p], e[p & 1]);
+                    }
+                    v[i] = (e[0] + e[1]) * r;
+                }
+            }
+        }
+        __syncthreads();
+        if (mine && lane < nb)
+#pragma unroll
+            for (int i = 0; i < NB; ++i)
+                if (i < nb && (low ? i > lane : i <= lane)) LU[(k0 + i) * ld + k0 + lane] = v[i];
+        __syncthreads();
+    }
+    // y <- U^-1 L^-1 y
+    auto solve = [&]() {
+        const int nblk = (n + NB - 1) / NB;
+        for (int t = 0; t < 2 * nblk; ++t) {
+            const bool fwd = t < nblk;
+            const int k0 = NB * (fwd ? t : 2 * nblk - 1 - t), nb = min(NB, n - k0);
+            if (warp == 0) {
+                // the block's solution by its inverse
+                float a0 = fwd && lane < nb ? y[k0 + lane] : 0.f, a1 = 0.f;
+                const float* inv = LU + (k0 + min(lane, nb - 1)) * ld + k0;
+#pragma unroll
+                for (int c = 0; c < NB; c += 2) {
+                    const bool u0 = fwd ? c < lane : c >= lane, u1 = fwd ? c + 1 < lane : c + 1 >= lane;
+                    a0 = fmaf(u0 && c < nb ? inv[c] : 0.f, y[k0 + c], a0);
+                    a1 = fmaf(u1 && c + 1 < nb ? inv[c + 1] : 0.f, y[k0 + c + 1], a1);
+                }
+                const float v = a0 + a1;
+                __syncwarp();
+                if (lane < nb) y[k0 + lane] = v;
+            }
+            __syncthreads();
+            const int i = tid;
+            if (i < n && (fwd ? i >= k0 + NB : i < k0)) {
+                float a0 = 0.f, a1 = 0.f;
+#pragma unroll 4
+                for (int p = 0; p < NB; p += 2) {
+                    if (p < nb) a0 = fmaf(LU[i * ld + k0 + p], y[k0 + p], a0);
+                    if (p + 1 < nb) a1 = fmaf(LU[i * ld + k0 + p + 1], y[k0 + p + 1], a1);
+                }
+                y[i] -= a0 + a1;
+            }
+            __syncthreads();
+        }
+    };
+    if (tid < n + 32) y[tid] = tid < n ? (float)b[tid] : 0.f;  // (the tail multiplies zeros)
+    __syncthreads();
+    solve();
+    if (tid < n) xs[tid] = (double)y[tid];
+    if (tid < 4) nrm[tid] = 0ull;
+    __syncthreads();
+    if (tid < n) {  // norms of A and b
+        atomicMax(&nrm[2], (unsigned long long)__double_as_longlong(ra[tid]));
+        atomicMax(&nrm[3], (unsigned long long)__double_as_longlong(fabs(b[tid])));
+    }
+    __syncthreads();
+    const double na = __longlong_as_double((long long)nrm[2]), nbv = __longlong_as_double((long long)nrm[3]);
+    double best = INFINITY;
+    for (int it = 0;; ++it) {
+        if (tid < 2) nrm[tid] = 0ull;
+        __syncthreads();
+        {
+            double s0 = 0.0, s1 = 0.0;
+            if (ri < n) {
+                const float* a = A + (size_t)ri * n;
+                int c = rh;
+#pragma unroll 4
+                for (; c + 2 < n; c += 4) s0 = fma((double)a[c], xs[c], s0), s1 = fma((double)a[c + 2], xs[c + 2], s1);
+                if (c < n) s0 = fma((double)a[c], xs[c], s0);
+                s0 += s1;
+            }
+            s0 += __shfl_xor_sync(0xffffffffu, s0, 1);
+            if (ri < n && rh == 0) {
+                const double r = b[ri] - s0, xi = xs[ri];
+                rs[ri] = r;
+                const double m = isfinite(r) && isfinite(xi) ? fabs(r) : INFINITY;
+                atomicMax(&nrm[0], (unsigned long long)__double_as_longlong(m));
+                atomicMax(&nrm[1], (unsigned long long)__double_as_longlong(fabs(xi)));
+            }
+        }
+        __syncthreads();
+        const double r = __longlong_as_double((long long)nrm[0]);
+        const double den = na * __longlong_as_double((long long)nrm[1]) + nbv;
+        const double be = den > 0.0 ? r / den : (r > 0.0 ? INFINITY : 0.0);
+        const bool done = be <= tol, last = it >= max_iter || !isfinite(be);
+        if (!done) {
+            if (be < best) {
+                best = be;
+                if (!last && tid < n) xb[tid] = xs[tid];
+            } else if (last && isfinite(best)) {
+                if (tid < n) xs[tid] = xb[tid];
+            }
+        }
+        if (done || last) {
+            if (tid < n) x[tid] = xs[tid];
+            if (tid == 0) out[0] = done ? 0.0 : 1.0, out[1] = (double)it, out[2] = done ? be : best;
+            return;
+        }
+        if (tid < n) y[tid] = (float)rs[tid];
+        __syncthreads();
+        solve();
+        if (tid < n) xs[tid] += (double)y[tid];
+    }
+}
+
 namespace {
 struct AicWs {
     size_t lu, t, perm, moves, info, dblk, dinv, pscratch, r, xbest, rowabs, norms, bytes;
@@ -1027,6 +1340,25 @@ vpm_status run_aic_solve(const float* A, const double* b, double* x, int n, doub
         const int reg_smem = PANEL_REG_ROWS * ((NB + 1) * sizeof(float) + 2 * sizeof(int));
         for (const void* f : reg_kernels)
             VPM_CU(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, reg_smem));
+    }
+    bool pivot_first = false;  // the small path has found that row exchanges are needed
+    if (n <= SMALL_N) {
+        VPM_CU(cudaFuncSetAttribute(aic_small_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    (int)small_smem(SMALL_N)));
+        trace_launch();
+        aic_small_kernel<<<1, SMALL_T, small_smem(n), st>>>(A, b, x, n, tol, max_iter, norms);
+        VPM_CU(cudaGetLastError());
+        double o[3];
+        VPM_CU(cudaMemcpyAsync(o, norms, sizeof(o), cudaMemcpyDeviceToHost, st));
+        VPM_CU(cudaStreamSynchronize(st));
+        if (o[0] < 2.0) {
+            if (iters) *iters = (int)o[1];
+            if (berr) *berr = o[2];
+            if (o[0] == 0.0) return VPM_OK;
+            *msg = "aic_solve: backward error above tol after max_iter refinement steps (best x written)";
+            return VPM_ERR_NOT_CONVERGED;
+        }
+        pivot_first = true;
     }
     const size_t solve_smem = (size_t)(n + SB) * sizeof(float);
     VPM_CU(cudaFuncSetAttribute(lu_solve_cluster_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -1134,10 +1466,15 @@ vpm_status run_aic_solve(const float* A, const double* b, double* x, int n, doub
         return e != cudaSuccess ? e : cudaGetLastError();
     };
     VPM_CU(cudaMemsetAsync(dflag, 0, sizeof(int), st));
-    trace_launch();
-    lu_dominance_kernel<<<(n * 32 + 255) / 256, 256, 0, st>>>(A, n, LU, dflag);
-    VPM_CU(factor(false));
-    bool pivoted = false;
+    bool pivoted = pivot_first;
+    if (pivot_first) {
+        VPM_CU(cudaMemcpyAsync(LU, A, (size_t)n * n * sizeof(float), cudaMemcpyDeviceToDevice, st));
+        VPM_CU(factor(true));
+    } else {
+        trace_launch();
+        lu_dominance_kernel<<<(n * 32 + 255) / 256, 256, 0, st>>>(A, n, LU, dflag);
+        VPM_CU(factor(false));
+    }
     double h[6];
     double best = INFINITY;
     for (int it = 0;; ++it) {
