@@ -164,9 +164,8 @@ vpm_status vpm_tree_induce(const float* pos_d, const float* str_d, int64_t n, fl
  * of vpm_segments_induce.  All sums accumulate in plain FP32 (VPM_COMPENSATED has no
  * effect here).  Vreman's eddy viscosity
  * and the stretching are formed in FP64 from the summed u and grad u (the transposed
- * stretching from J^T Gamma, not pair by pair), and the PSE term is summed over the
- * pairs within 7 sigma found by a walk of the same tree.  theta = 0 gives the direct
- * sums.  For particle counts where the direct sweep's O(n^2) cost dominates (1e6 and
+ * stretching from J^T Gamma, not pair by pair), and the PSE term is summed exactly, as
+ * in vpm_rhs, over the pairs within 7 sigma.  theta = 0 gives the direct sums.  For particle counts where the direct sweep's O(n^2) cost dominates (1e6 and
  * more).  Workspace: VPM_OP_RHS_TREE / VPM_OP_STEP_TREE (n_src = n, m_seg = m). */
 vpm_status vpm_rhs_tree(const float* pos_d, const float* str_d, int64_t n, const float* seg_a_d, const float* seg_b_d,
                         int64_t m, const vpm_params* prm, float theta, int order, float* dxdt_d, float* dGdt_d,
@@ -370,7 +369,9 @@ vpm_status vpm_wake_convert_row(const double* U_d, const double* D_d, const doub
  * The paper has no counterpart: this is a library convenience.  vpm_induce for
  * callers that cannot allocate device memory to pass as a workspace -- a solver in
  * C or Fortran linked without any CUDA memory manager, or a time-critical loop
- * that must not allocate.  Arguments and results are those of vpm_induce; the
+ * that must not allocate.  Arguments and results are those of vpm_induce (to rounding:
+ * it never uses the tensor cores, whose lists do not fit the scratch, so it takes about
+ * twice as long from some 16,000 particles on); the
  * scratch is a fixed VPM_NOALLOC_SCRATCH_BYTES array in the library's own device
  * memory, held by every GPU that loads the library until the process exits.
  *  - Every call looks the array's device address up on the current device; the
@@ -399,7 +400,8 @@ vpm_status vpm_induce_noalloc(const float* src_pos_d, const float* src_str_d, in
  * kind VPM_TRACE_ALL returns the total launch count of every kernel since the
  * last reset (and the summed time of all timed kinds).  Thread-safe. */
 #define VPM_TRACE_ALL 0
-#define VPM_TRACE_SWEEP 1     /* forward particle pair sweep with gradient (small problems: with the segments) */
+#define VPM_TRACE_SWEEP 1     /* forward particle pair sweep with gradient, its tensor-core and near launches
+                                 together (small problems: with the segments) */
 #define VPM_TRACE_ADJOINT 2   /* adjoint pair sweep */
 #define VPM_TRACE_PSE 3       /* particle strength exchange */
 #define VPM_TRACE_SWEEP_VEL 4 /* forward particle pair sweep, velocity only (the same) */

@@ -13,6 +13,12 @@
 // shared memory in 128-point tiles (bulk copies, double-buffered), work is split
 // stream-K over (particle tile, point tile) pairs and the partial sums are reduced
 // in a fixed order by a second kernel that also forms the outputs.
+//
+// The sums are also those of the forward sweep with the roles exchanged: with the
+// particles as targets and the points as sources of strength g_k, the velocity at particle
+// j is dL/dGamma_j and the transposed stretching J^T Gamma_j is dL/dx_j.  A problem large
+// enough for the tensor cores (FAR_MIN_UNITS_GRAD) runs so; adjoint_kernel
+// takes the smaller ones (1,280 points, 110,000 particles: 223 and 196 us).
 #include <algorithm>
 #include <math.h>
 

@@ -3,8 +3,10 @@
 //
 //  * aic_build: A[k][l] = u(ring l, unit circulation)(y_k) . n_k, each ring the four
 //    Vatistas-cored segments of its corners; b[k] = -(v_rel,k + w_k) . n_k in FP64.
-//  * aic_solve: A factored once in FP32 by a blocked right-looking LU with partial
-//    pivoting (panel kernel with one block barrier per column, row exchanges and the
+//  * aic_solve: orders up to 224 that are row-dominant in one launch of one block with
+//    the matrix in shared memory (aic_small_kernel); otherwise A is factored once in FP32
+//    by a blocked right-looking LU, without row exchanges if it is row-dominant and else
+//    with partial pivoting (panel kernel with one block barrier per column, row exchanges and the
 //    block row U12 in one kernel, FP32 update of the trailing matrix), then iterative
 //    refinement: the residual r = b - A x is formed in FP64 from the FP32 matrix, the
 //    correction solved with the FP32 factors (read through a transposed copy so that

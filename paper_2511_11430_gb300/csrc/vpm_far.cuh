@@ -18,8 +18,8 @@
 //
 // Bound and layout.  Per pair: 7 packed FP32 lanes' worth of FMA-pipe work and one rsqrt for
 // the weight, two conversions and a subtraction for its FP16 pair, one word of TMEM written;
-// the products (3 x 29 columns per pair) keep the tensor core a quarter busy.  The loop is
-// bound by issue slots and the FMA pipe (65% and 62% busy).  A thread owns two targets, one
+// the products (3 x 29 columns per pair) keep the tensor core a fifth busy.  The loop is
+// bound by issue slots and the FMA pipe (65% and 62% busy; the XU pipe 50%).  A thread owns two targets, one
 // row in each of two 128-row accumulators, and takes sources in pairs, so that a packed
 // register pair is one operand word and the source data is not duplicated; four warpgroups
 // per block work at their own pace on a shared ring of source tiles.  A chunk is 32 sources

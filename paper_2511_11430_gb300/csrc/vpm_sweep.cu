@@ -274,9 +274,11 @@ __host__ __device__ constexpr int n_rows()
 }
 
 
-// KIND: the source tiles a launch sweeps.  SWEEP_PARTICLES takes particle tiles and,
-// in the one-launch plan of small problems, segment tiles one segment at a time;
-// SWEEP_SEGMENTS takes only segment tiles, including those packed as closed rings.
+// KIND: the source tiles a launch sweeps.  SWEEP_SMALL (teams, below) takes particle tiles
+// and, where the segments are few, segment tiles one segment at a time; SWEEP_PARTICLES
+// takes the particle tiles of larger problems that have no tensor-core part (those without
+// a caller workspace, or beyond its unit limit).  SWEEP_SEGMENTS and SWEEP_SEG_SMALL take
+// only segment tiles, including those packed as closed rings.
 // The ring loop needs more registers than the particle loop; in a launch of its own
 // it costs the particle tiles nothing.  SWEEP_NEAR takes the particle tiles of a unit
 // list: those the tensor-core sweep (vpm_far.cuh) leaves.  They cluster (a source tile is

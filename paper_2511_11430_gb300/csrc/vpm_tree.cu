@@ -44,8 +44,8 @@
 // target leaf walks after the particle tree (far nodes into the same local expansion,
 // the others by the exact segment kernel); the summed u and grad u give Vreman's eddy
 // viscosity, the stretching and dx/dt per particle; the PSE term of Eq. 5 is then
-// summed by a second walk of the particle tree that visits only the nodes within
-// 7 sigma of each target leaf.
+// summed by the direct right-hand side's exchange kernel (vpm_sweep.cu) over tiles of
+// the particles in curve order.
 #include <math.h>
 
 #include <algorithm>
@@ -1303,7 +1303,7 @@ __global__ void tree_rhs_epilogue_kernel(int n, const float* __restrict__ up, co
     if (check && !isfinite(u[0] + u[1] + u[2] + st[0] + st[1] + st[2] + nut)) atomicOr(dev_err, DEV_ERR_NONFINITE);
 }
 
-// Sorted copies for the PSE walk: (x, y, z, volume) and (Gamma, nu_t).
+// Copies in curve order for the PSE: (x, y, z, volume) and (Gamma, nu_t).
 __global__ void tree_pse_gather_kernel(const float4* __restrict__ pos, const float4* __restrict__ str,
                                        const float* __restrict__ nu_t, const int* __restrict__ idx, int n,
                                        float4* __restrict__ sp, float4* __restrict__ sg, float* __restrict__ snut)
