@@ -588,8 +588,10 @@ def roofline(tr, n, m, sms, clk):
     # a small problem sweeps its segment tiles in the particle launch (no segment launch)
     flops_launch = FLOPS_P2P * n * (n - 1) + (FLOPS_SEG * n * m if not ns_ else 0)
     achieved = flops_launch / (avg_ms * 1e-3) / 1e12
+    kernel = ("far_sweep_kernel<grad, compensated> + sweep_kernel<grad, compensated, stretch, near>" if n >= 16384
+              else "sweep_kernel<grad, compensated, stretch, teams>")
     roof = {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "TFLOP/s", "frac": achieved / peak,
-            "traffic": sweep_traffic(n, m), "kernel": "far_sweep_kernel<grad, compensated> + sweep_kernel<grad, compensated, stretch, near>",
+            "traffic": sweep_traffic(n, m), "kernel": kernel,
             "launches": nl, "avg_launch_ms": avg_ms, "flops_per_launch": flops_launch,
             "peak_basis": f"{sms} SMs x 128 FP32 lanes x 2 (FFMA) x {sm_max:.0f} MHz max SM clock (derived)",
             "note": "flops of the direct pair form; the far tiles' products run on the tensor cores, so the rate can "
