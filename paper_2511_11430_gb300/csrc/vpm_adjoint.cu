@@ -16,7 +16,10 @@
 //
 // The sums are also those of the forward sweep with the roles exchanged: with the
 // particles as targets and the points as sources of strength g_k, the velocity at particle
-// j is dL/dGamma_j and the transposed stretching J^T Gamma_j is dL/dx_j.  A problem large
+// j is dL/dGamma_j and J^T Gamma_j is dL/dx_j, formed from the summed gradient.  (The sweep's
+// own stretching rows take near pairs with g_k - Gamma_j, which is exact when the two are
+// strengths of neighbours; here they are unrelated and g_k may be far smaller: dL/dx 1e-5
+// off at |g| = 1e-3 |Gamma| and 1e-2 off at 1e-6.)  A problem large
 // enough for the tensor cores (FAR_MIN_UNITS_GRAD) runs so; adjoint_kernel
 // takes the smaller ones (1,280 points, 110,000 particles: 223 and 196 us).
 #include <algorithm>
@@ -358,7 +361,7 @@ namespace {
 // computes at the particles: dL/dGamma = u (K r x g = K g x (x_j - y_k)) and dL/dx = J^T Gamma.
 // A problem large enough for the tensor cores takes that path (200,000 particles and 1,280
 // control points: 407 us by adjoint_kernel, 291 us so); a smaller one adjoint_kernel, which
-// accumulates 6 rows instead of 17 (60,000 particles: 170 against 185 us).
+// accumulates 6 rows instead of 14 (60,000 particles: 170 against 185 us).
 struct SweepAdj {
     SweepPlan p;
     size_t off_g, bytes;
@@ -368,7 +371,7 @@ SweepAdj plan_sweep_adjoint(int64_t n_src, int64_t n_tgt, bool comp)
 {
     Carve cv;
     SweepAdj a;
-    a.p = plan_sweep(n_src, n_tgt, 0, true, comp, cv, true);
+    a.p = plan_sweep(n_src, n_tgt, 0, true, comp, cv);
     a.off_g = cv.take((size_t)n_tgt * 16);
     a.bytes = cv.off;
     return a;

@@ -730,11 +730,12 @@ __global__ void __launch_bounds__(256) epilogue_kernel(const EpiArgs E)
         }
         return;
     }
-    if (o.mode == 2) {  // the adjoint at particle i
+    if (o.mode == 2) {  // the adjoint at particle i: u and J^T Gamma_i, the strength the target's own
+        const float4 G = reinterpret_cast<const float4*>(o.str)[i];
         o.dGdt[d] = (float)u0;
         o.dGdt[E.n + d] = (float)u1;
         o.dGdt[2 * E.n + d] = (float)u2;
-        for (int a = 0; a < 3; ++a) o.dxdt[(size_t)a * E.n + d] = (float)(acc[14 + a] * f4pi);
+        for (int a = 0; a < 3; ++a) o.dxdt[(size_t)a * E.n + d] = (float)(J[a] * G.x + J[3 + a] * G.y + J[6 + a] * G.z);
         return;
     }
     // Right-hand side of Eq. 4-5 for particle i.
