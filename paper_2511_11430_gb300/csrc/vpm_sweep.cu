@@ -731,7 +731,7 @@ __global__ void __launch_bounds__(256) epilogue_kernel(const EpiArgs E)
         return;
     }
     if (o.mode == 2) {  // the adjoint at particle i: u and J^T Gamma_i, the strength the target's own
-        const float4 G = reinterpret_cast<const float4*>(o.str)[i];
+        const float4 G = reinterpret_cast<const float4*>(o.str)[d];  // in the caller's order
         o.dGdt[d] = (float)u0;
         o.dGdt[E.n + d] = (float)u1;
         o.dGdt[2 * E.n + d] = (float)u2;
@@ -1124,7 +1124,7 @@ cudaError_t run_sweep(const SweepPlan& p, char* ws, const float* tgt, const floa
                                                          reinterpret_cast<const float4*>(src_str), p.n_src, perm, spos,
                                                          sstr, psrc, pbox);
     }
-    const float* own = out.str;
+    const float* own = out.str;  // the targets' own strengths, in the targets' order
     if (sorted) {
         tgt = src_pos = reinterpret_cast<const float*>(spos);
         src_str = reinterpret_cast<const float*>(sstr);
@@ -1246,7 +1246,7 @@ cudaError_t run_sweep(const SweepPlan& p, char* ws, const float* tgt, const floa
     E.ncomp = p.ncomp;
     E.comp = p.comp ? 1 : 0;
     E.o = out;
-    E.o.str = own;
+    if (out.mode != 2) E.o.str = own;  // (in the adjoint the sources' strengths are not the targets')
     E.perm = perm;
     E.dev_err = err;
     trace_launch();

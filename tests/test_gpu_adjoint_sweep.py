@@ -44,3 +44,19 @@ def test_loss_gradient_of_any_scale(api, scale):
     dx, dG = api.induce_backward(to_dev(w.pos), to_dev(w.strength), to_dev(pts), w.sigma, to_dev(g))
     assert api.device_error() == 0
     _check(dx, dG, w, pts, g, near)
+
+
+@pytest.mark.parametrize("n", [16_383, 16_384, 20_011])
+@pytest.mark.parametrize("alias", [True, False])
+def test_particles_as_their_own_points(api, n, alias):
+    """The points are the particles, in the same tensor or in a copy: in the first case the sweep puts sources
+    and targets in curve order, and the strengths that enter are still the particles', not the loss gradient."""
+    from paper_2511_11430_gb300 import autograd
+
+    w = synth.multirotor(seed=9, n=n)
+    P, S = to_dev(w.pos).requires_grad_(True), to_dev(w.strength).requires_grad_(True)
+    g = np.ascontiguousarray(np.random.default_rng(5).normal(size=(3, n)), dtype=np.float32)
+    u = autograd.induce(P, S, P.detach() if alias else P.detach().clone(), w.sigma)
+    dP, dS = torch.autograd.grad(u, (P, S), to_dev(g))
+    assert api.device_error() == 0
+    _check(dP[:, :3].t(), dS[:, :3].t(), w, w.pos, g)
