@@ -377,7 +377,7 @@ template <bool GRAD>
 __global__ void __launch_bounds__(LIST_TPB) far_mask_kernel(const float4* __restrict__ tgt, int n_tgt,
                                                             const unsigned char* __restrict__ tiles, int SP,
                                                             float far2, const float4* __restrict__ pbox,
-                                                            unsigned* __restrict__ mask, int2* __restrict__ cnt)
+                                                            unsigned* __restrict__ mask, uint2* __restrict__ cnt)
 {
     constexpr int GW = SWEEP_CW / FAR_GROUPS;  // warps per group
     __shared__ float wbox[SWEEP_CW][12];
@@ -439,40 +439,40 @@ __global__ void __launch_bounds__(LIST_TPB) far_mask_kernel(const float4* __rest
         }
     __syncthreads();
     const int KY = gridDim.y;
-    if (threadIdx.x == 0) cnt[(size_t)t * KY + blockIdx.y] = make_int2(tot[0][0], tot[0][1]);
+    if (threadIdx.x == 0) cnt[(size_t)t * KY + blockIdx.y] = make_uint2(tot[0][0], tot[0][1]);
     if (threadIdx.x < FAR_GROUPS)
         cnt[(size_t)gridDim.x * KY + ((size_t)t * FAR_GROUPS + threadIdx.x) * KY + blockIdx.y] =
-            make_int2(tot[1 + threadIdx.x][0], tot[1 + threadIdx.x][1]);
+            make_uint2(tot[1 + threadIdx.x][0], tot[1 + threadIdx.x][1]);
 }
 
 // Exclusive scans of the two count arrays, one per block.
-__global__ void __launch_bounds__(1024) far_scan_kernel(const int2* __restrict__ cnt, int m, int2* __restrict__ off_f,
-                                                        int2* __restrict__ off_n)
+__global__ void __launch_bounds__(1024) far_scan_kernel(const uint2* __restrict__ cnt, int m, uint2* __restrict__ off_f,
+                                                        uint2* __restrict__ off_n)
 {
-    __shared__ int2 ws[32];
+    __shared__ uint2 ws[32];
     const bool second = blockIdx.x != 0;
-    const int2* c = second ? cnt + m : cnt;
-    int2* off = second ? off_n : off_f;
+    const uint2* c = second ? cnt + m : cnt;
+    uint2* off = second ? off_n : off_f;
     const int len = second ? m * FAR_GROUPS : m;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    auto scan = [lane](int2 x) {
+    auto scan = [lane](uint2 x) {
         for (int o = 1; o < 32; o <<= 1) {
-            const int y0 = __shfl_up_sync(0xffffffffu, x.x, o), y1 = __shfl_up_sync(0xffffffffu, x.y, o);
+            const unsigned y0 = __shfl_up_sync(0xffffffffu, x.x, o), y1 = __shfl_up_sync(0xffffffffu, x.y, o);
             if (lane >= o) x.x += y0, x.y += y1;
         }
         return x;
     };
-    int2 base = make_int2(0, 0);
+    uint2 base = make_uint2(0, 0);
     for (int s = 0; s < len; s += 1024) {
         const int i = s + threadIdx.x;
-        const int2 own = i < len ? c[i] : make_int2(0, 0);
-        const int2 x = scan(own);
+        const uint2 own = i < len ? c[i] : make_uint2(0, 0);
+        const uint2 x = scan(own);
         if (lane == 31) ws[warp] = x;
         __syncthreads();
         if (warp == 0) ws[lane] = scan(ws[lane]);
         __syncthreads();
-        const int2 before = warp ? ws[warp - 1] : make_int2(0, 0);
-        if (i < len) off[i] = make_int2(base.x + before.x + x.x - own.x, base.y + before.y + x.y - own.y);
+        const uint2 before = warp ? ws[warp - 1] : make_uint2(0, 0);
+        if (i < len) off[i] = make_uint2(base.x + before.x + x.x - own.x, base.y + before.y + x.y - own.y);
         base.x += ws[31].x, base.y += ws[31].y;
         __syncthreads();
     }
@@ -481,15 +481,15 @@ __global__ void __launch_bounds__(1024) far_scan_kernel(const int2* __restrict__
 
 // blockIdx.z = 0: the tensor-core list of a (target tile, chunk); 1 + g: the pair sweep's of group g.
 __global__ void __launch_bounds__(LIST_TPB) far_emit_kernel(const unsigned* __restrict__ mask, int SP,
-                                                            const int2* __restrict__ off_f,
-                                                            const int2* __restrict__ off_n,
+                                                            const uint2* __restrict__ off_f,
+                                                            const uint2* __restrict__ off_n,
                                                             uint2* __restrict__ list_f, uint2* __restrict__ list_n)
 {
     constexpr int NW = LIST_TPB / 32;
-    __shared__ int2 ws[NW];
+    __shared__ uint2 ws[NW];
     const int t = blockIdx.x, g = (int)blockIdx.z - 1, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int k0 = blockIdx.y * FAR_KCH, k1 = min(SP, k0 + FAR_KCH);
-    int2 base = g < 0 ? off_f[t * gridDim.y + blockIdx.y] : off_n[(t * FAR_GROUPS + g) * gridDim.y + blockIdx.y];
+    uint2 base = g < 0 ? off_f[t * gridDim.y + blockIdx.y] : off_n[(t * FAR_GROUPS + g) * gridDim.y + blockIdx.y];
     uint2* list = g < 0 ? list_f : list_n;
     const unsigned lt = (1u << lane) - 1u;
     for (int ks = k0; ks < k1; ks += LIST_TPB) {
@@ -504,11 +504,11 @@ __global__ void __launch_bounds__(LIST_TPB) far_emit_kernel(const unsigned* __re
             const int y = __shfl_up_sync(0xffffffffu, s, o);
             if (lane >= o) s += y;
         }
-        if (lane == 31) ws[warp] = make_int2(__popc(q), s);
+        if (lane == 31) ws[warp] = make_uint2(__popc(q), s);
         __syncthreads();
-        int2 p = base;
+        uint2 p = base;
         for (int w = 0; w < NW; ++w) {
-            const int2 x = ws[w];
+            const uint2 x = ws[w];
             if (w < warp) p.x += x.x, p.y += x.y;
             base.x += x.x, base.y += x.y;
         }
@@ -520,8 +520,8 @@ __global__ void __launch_bounds__(LIST_TPB) far_emit_kernel(const unsigned* __re
 }
 
 cudaError_t run_far_lists(const float4* tgt, int n_tgt, const unsigned char* tiles, int SP, int TT, bool grad,
-                          const float4* pbox, float far2, unsigned* mask, int2* cnt, uint2* near_list, int2* near_off,
-                          uint2* far_list, int2* far_off, cudaStream_t st)
+                          const float4* pbox, float far2, unsigned* mask, uint2* cnt, uint2* near_list,
+                          uint2* near_off, uint2* far_list, uint2* far_off, cudaStream_t st)
 {
     const int KY = (SP + FAR_KCH - 1) / FAR_KCH;
     const dim3 grid(TT, KY), grid_emit(TT, KY, 1 + FAR_GROUPS);

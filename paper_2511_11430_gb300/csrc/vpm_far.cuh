@@ -78,27 +78,45 @@ struct FarTile {
 };
 constexpr size_t far_tile_bytes(bool grad) { return grad ? FarTile<true>::BYTES : FarTile<false>::BYTES; }
 
+// The cost line of a unit list, cut into equal ranges: at most B, each at least a whole unit
+// long, so that every range holds the start of one.  Costs are unsigned: a dense cloud in no
+// order at FAR_MAX_UNITS units costs 3.2e9.
+struct CostLine {
+    unsigned tot;
+    int B;
+    int max_cost;  // of one unit
+
+    __host__ __device__ __forceinline__ int blocks() const
+    {
+        const int whole = (int)(tot / (unsigned)max_cost);
+        return whole < 1 ? 1 : (whole < B ? whole : B);
+    }
+    // First cost of range b.
+    __host__ __device__ __forceinline__ long long begin(int b) const { return (long long)b * tot / blocks(); }
+    // Range owning the unit whose cost starts at c.
+    __host__ __device__ __forceinline__ int block_of(unsigned c) const
+    {
+        return (int)((((long long)c + 1) * blocks() - 1) / tot);
+    }
+};
+static_assert(FAR_MAX_UNITS * SWEEP_CW * NEAR_COST < (1LL << 32), "the pair sweep's costs fit 32 bits");
+static_assert(FAR_MAX_UNITS * (FAR_COST_FIRST + FAR_GROUPS - 1) < (1LL << 32), "the tensor-core sweep's costs fit 32 bits");
+static_assert(FAR_MAX_UNITS * FAR_GROUPS < (1LL << 31), "entry numbers fit 31 bits");
+
 // A list of units ordered by target tile: (source tile << 4 | group mask, cost of the
 // units before it); the pair sweep's is ordered by group and holds the source tile alone.
 // A unit's cost in the tensor-core list is far_cost of its groups, in the pair sweep's the
-// number of the group's warps, those within 7 sigma counted NEAR_COST times.  The cost line
-// is cut into equal ranges, one per block or team (at most B of them, and at least a whole
-// unit long, so that every range holds the start of one); block b runs the
-// units whose cost starts in its range and writes one partial sum per target tile into
-// slot b + t.
+// number of the group's warps, those within 7 sigma counted NEAR_COST times.  One block or
+// team runs the units whose cost starts in its range of the cost line and writes one partial
+// sum per target tile into slot b + t.
 struct UnitList {
     const uint2* list;
-    const int2* off;  // (entries, cost) before each (target tile, chunk); [TT * KY + 1]
+    const uint2* off;  // (entries, cost) before each (target tile, chunk); [TT * KY + 1]
     int TT, KY, B;
-    int max_cost;     // of one unit
+    int max_cost;      // of one unit
 
-    __device__ __forceinline__ int end(int t) const { return off[(t + 1) * KY].x; }
-    __device__ __forceinline__ int blocks(int tot) const { return max(1, min(B, tot / max_cost)); }
-    // Block owning the unit whose cost starts at c.
-    __device__ __forceinline__ int block_of(long long c, int tot) const
-    {
-        return (int)(((c + 1) * blocks(tot) - 1) / tot);
-    }
+    __device__ __forceinline__ int end(int t) const { return (int)off[(t + 1) * KY].x; }
+    __device__ __forceinline__ CostLine line() const { return CostLine{off[TT * KY].y, B, max_cost}; }
     // First index in [0, n) with key(index) >= v (n if none), key nondecreasing, by a whole warp:
     // 32 probes a round instead of one, since each round waits for memory.
     template <class Key>
@@ -120,15 +138,15 @@ struct UnitList {
     // The entries [lo, hi) of block b and the target tile of the first; by a whole warp.
     __device__ __forceinline__ void range(int b, int& lo, int& hi, int& t) const
     {
-        const int2 tot = off[TT * KY];
-        const int nb = blocks(tot.y);
+        const int entries = (int)off[TT * KY].x;
+        const CostLine cl = line();
         lo = hi = t = 0;
-        if (b >= nb) return;
+        if (b >= cl.blocks()) return;
         const uint2* l = list;
-        auto cost = [l](int q) { return (int)l[q].y; };
-        lo = warp_lower_bound(tot.x, (long long)b * tot.y / nb, cost);
-        hi = warp_lower_bound(tot.x, (long long)(b + 1) * tot.y / nb, cost);
-        const int2* o = off;
+        auto cost = [l](int q) { return l[q].y; };
+        lo = warp_lower_bound(entries, cl.begin(b), cost);
+        hi = warp_lower_bound(entries, cl.begin(b + 1), cost);
+        const uint2* o = off;
         const int ky = KY;
         t = warp_lower_bound(TT, (long long)lo + 1, [o, ky](int q) { return o[(q + 1) * ky].x; });
     }
@@ -146,8 +164,8 @@ struct FarArgs {
 cudaError_t run_far_pack(const float4* pos, const float4* str, int n, const float4* box, int SP, bool grad,
                          unsigned char* tiles, cudaStream_t st);
 cudaError_t run_far_lists(const float4* tgt, int n_tgt, const unsigned char* tiles, int SP, int TT, bool grad,
-                          const float4* pbox, float far2, unsigned* mask, int2* cnt, uint2* near_list, int2* near_off,
-                          uint2* far_list, int2* far_off, cudaStream_t st);
+                          const float4* pbox, float far2, unsigned* mask, uint2* cnt, uint2* near_list,
+                          uint2* near_off, uint2* far_list, uint2* far_off, cudaStream_t st);
 cudaError_t run_far_sweep(const FarArgs& A, bool grad, bool comp, cudaStream_t st);
 
 }  // namespace vpm

@@ -630,10 +630,10 @@ __global__ void __launch_bounds__(256) epilogue_kernel(const EpiArgs E)
     auto add_list = [&](const UnitList& ul, const float* part, int ncomp, auto ldc) {
         constexpr int ld = decltype(ldc)::value;
         const int t = min(i, E.n - 1) / ld, l = i % ld;
-        const int2 s = ul.off[t * ul.KY], e = ul.off[(t + 1) * ul.KY];
+        const uint2 s = ul.off[t * ul.KY], e = ul.off[(t + 1) * ul.KY];
         if (s.x >= e.x) return;
-        const int tot = ul.off[ul.TT * ul.KY].y;
-        const int b0 = ul.block_of(s.y, tot), b1 = ul.block_of(ul.list[e.x - 1].y, tot), rows = E.comp ? 2 * ncomp : ncomp;
+        const CostLine cl = ul.line();
+        const int b0 = cl.block_of(s.y), b1 = cl.block_of(ul.list[e.x - 1].y), rows = E.comp ? 2 * ncomp : ncomp;
         for (int b = b0 + part_i; b <= b1; b += PARTS) add(part + (size_t)(b + t) * rows * ld + l, ncomp, ldc);
     };
     if (E.far) {
@@ -1061,11 +1061,11 @@ SweepPlan plan_sweep(int64_t n_tgt, int64_t n_src, int64_t m_seg, bool grad, boo
         const size_t rows_f = (size_t)(comp ? 2 : 1) * (grad ? 14 : 3);
         p.off_ftile = cv.take((size_t)p.SP * far_tile_bytes(grad));
         p.off_fmask = cv.take((size_t)units * sizeof(unsigned));
-        p.off_fcnt = cv.take((size_t)p.TT * p.KY * (1 + FAR_GROUPS) * sizeof(int2));
+        p.off_fcnt = cv.take((size_t)p.TT * p.KY * (1 + FAR_GROUPS) * sizeof(uint2));
         p.off_nlist = cv.take((size_t)units * FAR_GROUPS * sizeof(uint2));
-        p.off_noff = cv.take(((size_t)p.TT * p.KY * FAR_GROUPS + 1) * sizeof(int2));
+        p.off_noff = cv.take(((size_t)p.TT * p.KY * FAR_GROUPS + 1) * sizeof(uint2));
         p.off_flist = cv.take((size_t)units * sizeof(uint2));
-        p.off_foff = cv.take(((size_t)p.TT * p.KY + 1) * sizeof(int2));
+        p.off_foff = cv.take(((size_t)p.TT * p.KY + 1) * sizeof(uint2));
         p.off_part_f = cv.take((size_t)(p.TT + p.B_far) * rows_f * TGT_TILE * sizeof(float));
         constexpr int teams = Ring<SWEEP_NEAR>::TEAMS;
         p.off_part_n = cv.take((size_t)(p.TT * FAR_GROUPS + p.B_near * teams) * rows * FAR_GROUP * sizeof(float));
@@ -1143,7 +1143,7 @@ cudaError_t run_sweep(const SweepPlan& p, char* ws, const float* tgt, const floa
         auto list = [&](size_t l, size_t o, int T, int B, int max_cost) {
             UnitList u;
             u.list = reinterpret_cast<const uint2*>(ws + l);
-            u.off = reinterpret_cast<const int2*>(ws + o);
+            u.off = reinterpret_cast<const uint2*>(ws + o);
             u.TT = T;
             u.KY = p.KY;
             u.B = B;
@@ -1159,9 +1159,9 @@ cudaError_t run_sweep(const SweepPlan& p, char* ws, const float* tgt, const floa
             e = run_far_lists(reinterpret_cast<const float4*>(tgt), p.n_tgt, ftile, p.SP, p.TT, p.grad, pbox,
                               (float)((double)RHO_FAR * RHO_FAR * (double)sigma * (double)sigma),
                               reinterpret_cast<unsigned*>(ws + p.off_fmask),
-                              reinterpret_cast<int2*>(ws + p.off_fcnt), reinterpret_cast<uint2*>(ws + p.off_nlist),
-                              reinterpret_cast<int2*>(ws + p.off_noff), reinterpret_cast<uint2*>(ws + p.off_flist),
-                              reinterpret_cast<int2*>(ws + p.off_foff), st);
+                              reinterpret_cast<uint2*>(ws + p.off_fcnt), reinterpret_cast<uint2*>(ws + p.off_nlist),
+                              reinterpret_cast<uint2*>(ws + p.off_noff), reinterpret_cast<uint2*>(ws + p.off_flist),
+                              reinterpret_cast<uint2*>(ws + p.off_foff), st);
         if (e != cudaSuccess) return e;
     }
     if (p.SP + p.SS > 0) {
