@@ -275,14 +275,17 @@ __global__ void __launch_bounds__(SRC_TILE) far_pack_kernel(const float4* __rest
     __syncthreads();
     for (int w = 0; w < SRC_TILE / 32; ++w) r2 = fmaxf(r2, red[0][w]), gm = fmaxf(gm, red[1][w]);
     const float rad = sqrtf(r2) * 1.000001f;
-    // scales: powers of two above the radius and the largest strength component, so that
-    // the scaled values are exact
+    // scales: powers of two above the radius and the largest strength component, so that the
+    // scaled values are exact (strengths at most 2^FAR_FEXP; eg is kept where both its
+    // scale and the inverse are normal numbers)
     int ea = 0, eg = 0;
     frexpf(rad, &ea);
     frexpf(gm, &eg);
-    const bool tiny = !(rad > 1e-30f), weak = !(gm > 1e-30f);
-    const float a = tiny || any_bad ? 1.f : ldexpf(1.f, ea), gam = weak || any_bad ? 1.f : ldexpf(1.f, eg);
-    const float ia = 1.f / a, ig = FAR_FSCALE / gam;
+    eg = max(eg, FAR_FEXP - 126);
+    const bool tiny = !(rad > 1e-30f);
+    const float a = tiny || any_bad ? 1.f : ldexpf(1.f, ea);
+    const float gam = any_bad ? 1.f : ldexpf(1.f, eg - FAR_FEXP), ig = any_bad ? 1.f : ldexpf(1.f, FAR_FEXP - eg);
+    const float ia = 1.f / a;
     const float x = d[0] * ia, y = d[1] * ia, z = d[2] * ia, q = x * x + y * y + z * z;
     const float gx = G[0] * ig, gy = G[1] * ig, gz = G[2] * ig;
     const float mx = gy * z - gz * y, my = gz * x - gx * z, mz = gx * y - gy * x;  // Gamma x d
@@ -332,7 +335,7 @@ __global__ void __launch_bounds__(SRC_TILE) far_pack_kernel(const float4* __rest
         if (s == 0 && i < T::N) hdr[i] = v + w;
     }
     if (tid < 8) {
-        const float v[8] = {c[0], c[1], c[2], a, gam / FAR_FSCALE, any_bad ? INFINITY : rad, 0.f, 0.f};
+        const float v[8] = {c[0], c[1], c[2], a, gam, any_bad ? INFINITY : rad, 0.f, 0.f};
         hdr[T::N + tid] = v[tid];
     }
     for (int i = T::N + 8 + tid; i < 64; i += SRC_TILE) hdr[i] = 0.f;

@@ -63,7 +63,7 @@ constexpr long long FAR_MAX_UNITS = 1LL << 26;   // ... and to which (the unit l
 // 611 and 638 us; hover wake 679 and 690 us, 488 and 572 us).
 constexpr int FAR_SORT_MIN = 16384;
 constexpr int FAR_KCH = 2048;                    // source tiles per block of the mask and list kernels
-constexpr float FAR_FSCALE = 256.f;              // features are scaled by this before their FP16 split
+constexpr int FAR_FEXP = 8;                      // features are scaled to at most 2^8 before their FP16 split
 
 // Packed far tile: FP16 features hi then lo in the tensor core's K-major core-matrix
 // order, the scaled offsets in source pairs, the header.
