@@ -265,7 +265,8 @@ __global__ void __launch_bounds__(SRC_TILE) far_pack_kernel(const float4* __rest
         G[0] = s.x, G[1] = s.y, G[2] = s.z;
     }
     float r2 = d[0] * d[0] + d[1] * d[1] + d[2] * d[2], gm = fmaxf(fabsf(G[0]), fmaxf(fabsf(G[1]), fabsf(G[2])));
-    const bool bad = !isfinite(r2) || !isfinite(G[0]) || !isfinite(G[1]) || !isfinite(G[2]);
+    const bool bad = !isfinite(r2) || !isfinite(G[0]) || !isfinite(G[1]) || !isfinite(G[2]) ||
+                     !(fmaxf(fabsf(c[0]), fmaxf(fabsf(c[1]), fabsf(c[2]))) < FAR_XMAX);
     const bool any_bad = __syncthreads_or(bad) != 0;
     for (int o = 16; o > 0; o >>= 1) {
         r2 = fmaxf(r2, __shfl_xor_sync(0xffffffffu, r2, o));
@@ -385,6 +386,7 @@ __global__ void __launch_bounds__(LIST_TPB) far_mask_kernel(const float4* __rest
     constexpr int GW = SWEEP_CW / FAR_GROUPS;  // warps per group
     __shared__ float wbox[SWEEP_CW][12];
     __shared__ int tot[1 + FAR_GROUPS][2];
+    __shared__ int beyond[SWEEP_CW];  // a target of the warp lies beyond FAR_XMAX (or is not finite)
     const int t = blockIdx.x, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (threadIdx.x < 2 * (1 + FAR_GROUPS)) (&tot[0][0])[threadIdx.x] = 0;
     const int i0 = t * TGT_TILE + warp * 64 + lane, i1 = i0 + 32;
@@ -393,6 +395,9 @@ __global__ void __launch_bounds__(LIST_TPB) far_mask_kernel(const float4* __rest
     if (v0) p0 = tgt[i0];
     if (v1) p1 = tgt[i1];
     warp_two_boxes(make_float3(p0.x, p0.y, p0.z), v0, make_float3(p1.x, p1.y, p1.z), v1, wbox[warp]);
+    auto inside = [](float4 p) { return fabsf(p.x) < FAR_XMAX && fabsf(p.y) < FAR_XMAX && fabsf(p.z) < FAR_XMAX; };
+    const bool all_in = __all_sync(0xffffffffu, inside(p0) && inside(p1));  // (a lane without a target holds zeros)
+    if (lane == 0) beyond[warp] = !all_in;
     __syncthreads();
     const int k0 = blockIdx.y * FAR_KCH, k1 = min(SP, k0 + FAR_KCH);
     int v[1 + FAR_GROUPS][2] = {};
@@ -400,7 +405,7 @@ __global__ void __launch_bounds__(LIST_TPB) far_mask_kernel(const float4* __rest
         const float4* h = reinterpret_cast<const float4*>(tiles + (size_t)k * FarTile<GRAD>::BYTES +
                                                           FarTile<GRAD>::OFF_H + FarTile<GRAD>::N * 4);
         const float4 c = h[0];  // centre, scale
-        const float rad = h[1].y;  // radius; +inf for a tile with a non-finite source
+        const float rad = h[1].y;  // radius; +inf for a tile with a non-finite source or beyond FAR_XMAX
         const float sep = rad + sqrtf(far2) * 1.0001f;
         const float need = fmaxf(rad * (1.f / FAR_TAU), sep), need2 = need * need;
         const float4 tlo = pbox[2 * k], thi = pbox[2 * k + 1];
@@ -408,6 +413,8 @@ __global__ void __launch_bounds__(LIST_TPB) far_mask_kernel(const float4* __rest
 #pragma unroll
         for (int g = 0; g < FAR_GROUPS; ++g) {
             bool far = true;
+#pragma unroll
+            for (int w = g * GW; w < (g + 1) * GW; ++w) far = far && !beyond[w];
 #pragma unroll 1
             for (int w = g * GW; w < (g + 1) * GW; ++w)
 #pragma unroll

@@ -62,6 +62,9 @@ constexpr long long FAR_MAX_UNITS = 1LL << 26;   // ... and to which (the unit l
 // side of the BVI wake: 16,000 particles 819 us without and 744 us with it, 12,000 particles
 // 611 and 638 us; hover wake 679 and 690 us, 488 and 572 us).
 constexpr int FAR_SORT_MIN = 16384;
+// Coordinates up to which |x - y|^2 stays finite in FP32.  Beyond, a pair contributes nothing
+// in the pair sweep (1/r of an infinite r^2), which takes the groups and tiles concerned.
+constexpr float FAR_XMAX = 4e18f;
 constexpr int FAR_KCH = 2048;                    // source tiles per block of the mask and list kernels
 constexpr int FAR_FEXP = 8;                      // features are scaled to at most 2^8 before their FP16 split
 

@@ -40,3 +40,16 @@ def test_strengths_of_any_size(api, size):
     w = synth.hover(seed=5, n=60_000)
     G = np.float32(w.strength * (size / 1e-3))
     _check(api, w.pos, G, w.pos, w.sigma, synth.sample_targets(5, w.n, 96))
+
+
+@pytest.mark.parametrize("d", [1e18, 3e19, 1e30, 1e37])
+@pytest.mark.parametrize("which", ["sources", "targets", "both"])
+def test_distances_whose_squares_overflow(api, d, which):
+    """200 particles so far off that r^2 is not finite in FP32 (from 1.8e19): they contribute nothing to the
+    others and the others nothing to them."""
+    w = synth.hover(seed=5, n=60_000)
+    off = w.pos.copy()
+    off[:200, 0] += np.float32(d)
+    src, tgt = (w.pos if which == "targets" else off), (w.pos if which == "sources" else off)
+    idx = np.concatenate([np.arange(0, 200, 20), 200 + synth.sample_targets(5, w.n - 200, 96)])
+    _check(api, src, w.strength, tgt, w.sigma, idx)
