@@ -164,11 +164,11 @@ __device__ __forceinline__ void near_kh2(f2 r2, const NearConst& nc, f2& K, f2& 
     e = fma2(mul2(e, splat(0.69314718f)), lo, e);
     const f2 q = fma2(w, Fw, mul2(e, splat(0.26596152026762182f)));  // sqrt(2/pi)/3
     const f2 Kn = mul2(q, splat(nc.inv_s3)), hn = mul2(Fw, splat(nc.inv_s5));
-    // a pair at zero distance contributes nothing (its h multiplies zero vectors)
+    // a pair at zero distance contributes nothing (its h too: sigma^-5 overflows from 2e-8 down)
     K.x = r2.x < nc.far2 ? (r2.x == 0.f ? 0.f : Kn.x) : Kf.x;
     K.y = r2.y < nc.far2 ? (r2.y == 0.f ? 0.f : Kn.y) : Kf.y;
-    h.x = r2.x < nc.far2 ? hn.x : hf.x;
-    h.y = r2.y < nc.far2 ? hn.y : hf.y;
+    h.x = r2.x < nc.far2 ? (r2.x == 0.f ? 0.f : hn.x) : hf.x;
+    h.y = r2.y < nc.far2 ? (r2.y == 0.f ? 0.f : hn.y) : hf.y;
 }
 
 // ---------------------------------------------------------------------------

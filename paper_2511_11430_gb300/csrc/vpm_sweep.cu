@@ -28,6 +28,7 @@
 // tensor cores instead (vpm_far.cuh), over particles in curve order.  Each tile's sums start from zero and are folded into a
 // per-thread running sum kept in shared memory: a compensated (hi, lo) pair with
 // Knuth's two-sum, or a plain sum, so long source lists keep a tile-sized error.
+#include <float.h>
 #include <math.h>
 
 #include <algorithm>
@@ -1087,6 +1088,12 @@ SweepPlan plan_sweep(int64_t n_tgt, int64_t n_src, int64_t m_seg, bool grad, boo
     return p;
 }
 
+// (7 sigma)^2, above zero for any core: a pair at zero distance is near, and contributes nothing.
+static float far2_of(float sigma)
+{
+    return std::max((float)((double)RHO_FAR * RHO_FAR * (double)sigma * (double)sigma), FLT_MIN);
+}
+
 template <bool G, bool C, bool S>
 static void launch_sweep(const SweepArgs& A, int B, int kind, cudaStream_t st)
 {
@@ -1162,7 +1169,7 @@ cudaError_t run_sweep(const SweepPlan& p, char* ws, const float* tgt, const floa
                                      p.n_src, pbox, p.SP, p.grad, reinterpret_cast<unsigned char*>(ws + p.off_ftile), st);
         if (e == cudaSuccess)
             e = run_far_lists(reinterpret_cast<const float4*>(tgt), p.n_tgt, ftile, p.SP, p.TT, p.grad, pbox,
-                              (float)((double)RHO_FAR * RHO_FAR * (double)sigma * (double)sigma),
+                              far2_of(sigma),
                               reinterpret_cast<unsigned*>(ws + p.off_fmask),
                               reinterpret_cast<uint2*>(ws + p.off_fcnt), reinterpret_cast<uint2*>(ws + p.off_nlist),
                               reinterpret_cast<uint2*>(ws + p.off_noff), reinterpret_cast<uint2*>(ws + p.off_flist),
@@ -1190,7 +1197,7 @@ cudaError_t run_sweep(const SweepPlan& p, char* ws, const float* tgt, const floa
         A.nc.inv_s2 = (float)(1.0 / (s * s));
         A.nc.inv_s3 = (float)(1.0 / (s * s * s));
         A.nc.inv_s5 = (float)(1.0 / (s * s * s * s * s));
-        A.nc.far2 = (float)((double)RHO_FAR * RHO_FAR * s * s);
+        A.nc.far2 = far2_of(sigma);
         A.dev_err = err;
         for (int kind = 0; kind < 2; ++kind) {
             const bool seg = kind == 1;

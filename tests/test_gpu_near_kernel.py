@@ -42,3 +42,28 @@ def test_single_pairs(sigma, compensated):
     dJ = np.abs(g.double().cpu().numpy().T.reshape(-1, 3, 3) - rJ).max((1, 2))
     assert (dJ / (2 * K * np.linalg.norm(G[0, :3]))).max() <= TOL_J
     assert api.device_error() == 0
+
+
+@pytest.mark.parametrize("n", [300, 17_003])
+@pytest.mark.parametrize("sigma", [1e-6, 1e-9, 1e-15, 1e-25])
+def test_point_vortices(sigma, n):
+    """Cores so small that sigma^-5, sigma^-3 or sigma^2 leave FP32: point vortices, none of which acts on itself
+    or on one in the same place."""
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2511_11430_gb300 import api, build, synth
+    from tests._util import TOL_COMP, rel_l2
+
+    build.build()
+    w = synth.hover(seed=2, n=n)
+    pos = w.pos.copy()
+    pos[10:20, :3] = pos[10, :3]
+    idx = np.unique(np.concatenate([np.arange(8, 22), synth.sample_targets(5, n, 96)]))
+    P, S = to_dev(pos), to_dev(w.strength)
+    u, g = api.induce(P, S, P, sigma)
+    uv = api.induce(P, S, P, sigma, grad=False)
+    ru, rJ = oracle.p2p(pos, w.strength, pos[idx], sigma)
+    rows = lambda t: t[:, idx].double().cpu().numpy().T
+    assert rel_l2(rows(u), ru) <= TOL_COMP and rel_l2(rows(uv), ru) <= TOL_COMP
+    assert rel_l2(rows(g).reshape(-1, 3, 3), rJ) <= TOL_COMP
+    assert api.device_error() == 0
