@@ -426,13 +426,16 @@ __global__ void __launch_bounds__(LIST_TPB) far_mask_kernel(const float4* __rest
                     far = far && dx * dx + dy * dy + dz * dz > need2;
                 }
             int cn = 0;
-            if (t * TGT_TILE + g * FAR_GROUP >= n_tgt)
+            const int warps = group_warps(n_tgt - (t * TGT_TILE + g * FAR_GROUP));
+            if (warps == 0)
                 ;  // no target: in neither list
             else if (far)
                 m |= 1u << g;
-            else
+            else {
 #pragma unroll 1
-                for (int w = g * GW; w < (g + 1) * GW; ++w) cn += boxes_near(wbox[w], tlo, thi, far2) ? NEAR_COST : 1;
+                for (int w = g * GW; w < g * GW + warps; ++w) cn += boxes_near(wbox[w], tlo, thi, far2) ? NEAR_COST : 1;
+                cn = ragged_cost(cn, warps);
+            }
             m |= (unsigned)cn << (8 + 6 * g);
             v[1 + g][0] += cn != 0, v[1 + g][1] += cn;
         }

@@ -58,6 +58,17 @@ int main()
     // tensor-core sweep: all groups of every unit
     for (long long units : {1LL, 151LL, 2049LL, FAR_MAX_UNITS})
         bad |= check("far", units, FAR, 152, [](long long) { return FAR; });
+    // a ragged group's unit costs what a whole group's costs when its warps are alike, and no
+    // more than the dearest
+    for (int left = -3; left <= FAR_GROUP + 70; ++left) {
+        const int w = group_warps(left);
+        if (w != (left <= 0 ? 0 : left > 192 ? 4 : left > 128 ? 3 : left > 64 ? 2 : 1)) bad = 1, printf("warps of %d targets: %d\n", left, w);
+        for (int near = 0; w > 0 && near <= w; ++near) {
+            const int c = ragged_cost(near * NEAR_COST + (w - near), w);
+            if (c < WARPS || c > NEAR || (near == 0 && c != WARPS) || (near == w && c != NEAR))
+                bad = 1, printf("ragged cost of %d warps, %d near: %d\n", w, near, c);
+        }
+    }
     if (!bad) printf("OK\n");
     return bad;
 }
