@@ -58,14 +58,15 @@ __device__ __forceinline__ void particle_tile(Acc<GRAD, STRETCH>& a, const float
     }
 }
 
-// The sources of a particle tile selected by `keep` (bit j of keep[h]: source 32 h + j).
+// The sources of a particle tile selected by `keep` (bit j of keep[h]: source 32 h + j), words
+// h0 to h1.
 template <bool GRAD, bool STRETCH, bool NEAR>
 __device__ __forceinline__ void particle_subset(Acc<GRAD, STRETCH>& a, const float4* __restrict__ s,
-                                                const unsigned (&keep)[SRC_TILE / 32], bool invert, int cnt, f2 X,
-                                                f2 Y, f2 Z, const NearConst& nc, const Own& o)
+                                                const unsigned (&keep)[SRC_TILE / 32], int h0, int h1, bool invert,
+                                                int cnt, f2 X, f2 Y, f2 Z, const NearConst& nc, const Own& o)
 {
 #pragma unroll 1
-    for (int h = 0; 32 * h < cnt; ++h) {
+    for (int h = h0; h < h1 && 32 * h < cnt; ++h) {
         unsigned m = h == 0 ? keep[0] : h == 1 ? keep[1] : h == 2 ? keep[2] : keep[3];
         const int left = cnt - 32 * h;
         if (invert) m = ~m & (left >= 32 ? 0xffffffffu : (1u << left) - 1u);
@@ -431,6 +432,19 @@ __global__ void __launch_bounds__(SWEEP_TPB, 1) sweep_kernel(const SweepArgs A)
         for (int q = 0; q < NR * (COMP ? 2 : 1); ++q) run[q * NT + ct] = zero2();
     };
     zero_run();
+    auto fold_acc = [&]() {  // the sums of a tile (or half of one) into the running sums
+#pragma unroll
+        for (int q = 0; q < NR; ++q) {
+            if (COMP) {
+                f2 hi = run[(2 * q) * NT + ct], lo = run[(2 * q + 1) * NT + ct];
+                fold2(hi, lo, acc.v[q]);
+                run[(2 * q) * NT + ct] = hi;
+                run[(2 * q + 1) * NT + ct] = lo;
+            } else {
+                run[q * NT + ct] = add2(run[q * NT + ct], acc.v[q]);
+            }
+        }
+    };
     for (int i = 0;; ++i) {
         const int s = s0 + i % R::STAGES, r = i / R::STAGES;
         int nt = t, nk = k + 1;
@@ -475,13 +489,23 @@ __global__ void __launch_bounds__(SWEEP_TPB, 1) sweep_kernel(const SweepArgs A)
         // stretching from the tile's sums afterwards.  Near particle tiles accumulate the
         // stretching pair by pair (it cancels there) with the strengths loaded for them.
         const int ti0 = t * R::TGT + (warp % R::WARPS) * 64 + lane, ti1 = ti0 + 32;
+        // Near sources summed in a row.  In curve order a target's neighbours fill whole tiles, and the
+        // rounding of their sums grows with the run, where in the caller's order they were spread over
+        // many tiles; halved, it is below what it was there (20,011-particle hover wake, error of nu_t:
+        // 8.9e-7 in the caller's order, 9.8e-7 in curve order and whole tiles, 7.1e-7 in halves; 886
+        // and 884 us a right-hand side).
+        constexpr int NEAR_RUN = LIST && COMP && GRAD ? SRC_TILE / 2 : R::UNIT;
         if (LIST || (!R::SEG && k < sk.np)) {
             const int cnt = min(R::UNIT, A.n_src - k * R::UNIT);  // (the last half tile may be empty)
             const float4 tlo = src[R::BOX], thi = src[R::BOX + 1];
             if (boxes_near(wbox[warp], tlo, thi, A.nc.far2)) {
                 if constexpr (!STRETCH) {
-                    acc.zero();
-                    particle_tile<GRAD, false, true>(acc, src, cnt, X, Y, Z, A.nc, Own{});
+                    for (int j = 0;; j += NEAR_RUN) {
+                        acc.zero();
+                        particle_tile<GRAD, false, true>(acc, src + j * P_F4, min(NEAR_RUN, cnt - j), X, Y, Z, A.nc, Own{});
+                        if (j + NEAR_RUN >= cnt) break;
+                        fold_acc();
+                    }
                 } else {
                     Own own;
                     float4 g0 = make_float4(0.f, 0.f, 0.f, 0.f), g1 = g0;
@@ -505,10 +529,16 @@ __global__ void __launch_bounds__(SWEEP_TPB, 1) sweep_kernel(const SweepArgs A)
                     {
                         Acc<GRAD, false> tf;
                         tf.zero();
-                        particle_subset<GRAD, false, false>(tf, src, keep, true, cnt, X, Y, Z, A.nc, Own{});
+                        particle_subset<GRAD, false, false>(tf, src, keep, 0, SRC_TILE / 32, true, cnt, X, Y, Z, A.nc, Own{});
                         finish_tile<GRAD, STRETCH>(acc, tf, A.tstr, ti0, ti1, A.n_tgt);
                     }
-                    particle_subset<GRAD, true, true>(acc, src, keep, false, cnt, X, Y, Z, A.nc, own);
+                    particle_subset<GRAD, true, true>(acc, src, keep, 0, NEAR_RUN / 32, false, cnt, X, Y, Z, A.nc, own);
+                    if (NEAR_RUN < SRC_TILE && (keep[2] | keep[3])) {
+                        fold_acc();
+                        acc.zero();
+                        particle_subset<GRAD, true, true>(acc, src, keep, NEAR_RUN / 32, SRC_TILE / 32, false, cnt, X, Y, Z, A.nc,
+                                                          own);
+                    }
                 }
             } else {
                 Acc<GRAD, false> tf;
@@ -545,18 +575,7 @@ __global__ void __launch_bounds__(SWEEP_TPB, 1) sweep_kernel(const SweepArgs A)
                 if (unit_ahead(i, t, k, R::STAGES, kk)) issue(kk, s, r + 1);
             }
         }
-        // fold this tile's sums into the running sums
-#pragma unroll
-        for (int q = 0; q < NR; ++q) {
-            if (COMP) {
-                f2 hi = run[(2 * q) * NT + ct], lo = run[(2 * q + 1) * NT + ct];
-                fold2(hi, lo, acc.v[q]);
-                run[(2 * q) * NT + ct] = hi;
-                run[(2 * q + 1) * NT + ct] = lo;
-            } else {
-                run[q * NT + ct] = add2(run[q * NT + ct], acc.v[q]);
-            }
-        }
+        fold_acc();
         if (!has_next || nt != t) {  // this warp's partial of target tile (LIST: group) t
             float* P = A.part + ((size_t)(b + t) * (COMP ? 2 * NR : NR)) * R::TGT + (warp % R::WARPS) * 64 + lane;
 #pragma unroll
