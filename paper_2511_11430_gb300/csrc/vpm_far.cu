@@ -124,9 +124,16 @@ __device__ __forceinline__ void far_weight(f2 t, uint32_t& hi, uint32_t& neg)
 // a Hilbert curve they are compact, and so are the target groups.  (Morton order leaves
 // jumps: on the 20,000-particle hover wake 74% of the pairs pass the acceptance test in
 // Morton order, 80% in Hilbert order and 1% in the generator's filament order.)
-// 8 bits per axis: three radix passes, and cells far smaller than a tile.
+// 8 bits per axis: three radix passes, and cells far smaller than a tile.  Where the cost of a
+// poor order grows with the square of the count (the treecode's exchange), 21 bits: a stray
+// particle a thousand wake lengths away leaves the rest in a few of the coarse cells, in the
+// caller's order (1,000,000 particles in no order, right-hand side: 531 ms, with the fine cells 31).
 // ---------------------------------------------------------------------------
-constexpr int CURVE_BITS = 8;
+template <bool FINE>
+struct Curve {
+    using Key = typename std::conditional<FINE, unsigned long long, unsigned>::type;
+    static constexpr int BITS = FINE ? 21 : 8;
+};
 constexpr int CURVE_BND_BLOCKS = 128;  // partial boxes of the curve's bounding cube
 
 __global__ void __launch_bounds__(256) curve_bounds_kernel(const float4* __restrict__ pos, int n, float* __restrict__ bnd)
@@ -153,11 +160,13 @@ __global__ void __launch_bounds__(256) curve_bounds_kernel(const float4* __restr
 
 // Position along the Hilbert curve of a cell (Skilling, "Programming the Hilbert curve",
 // AIP Conf. Proc. 707, 2004: the transpose form).
-__device__ __forceinline__ unsigned hilbert_key(unsigned x, unsigned y, unsigned z)
+template <bool FINE>
+__device__ __forceinline__ typename Curve<FINE>::Key hilbert_key(unsigned x, unsigned y, unsigned z)
 {
+    constexpr int BITS = Curve<FINE>::BITS;
     unsigned X[3] = {x, y, z};
 #pragma unroll
-    for (unsigned Q = 1u << (CURVE_BITS - 1); Q > 1; Q >>= 1) {
+    for (unsigned Q = 1u << (BITS - 1); Q > 1; Q >>= 1) {
         const unsigned P = Q - 1;
 #pragma unroll
         for (int i = 0; i < 3; ++i) {
@@ -174,20 +183,23 @@ __device__ __forceinline__ unsigned hilbert_key(unsigned x, unsigned y, unsigned
     X[2] ^= X[1];
     unsigned t = 0;
 #pragma unroll
-    for (unsigned Q = 1u << (CURVE_BITS - 1); Q > 1; Q >>= 1)
+    for (unsigned Q = 1u << (BITS - 1); Q > 1; Q >>= 1)
         if (X[2] & Q) t ^= Q - 1;
-    unsigned k = 0;
+    typename Curve<FINE>::Key k = 0;
 #pragma unroll
-    for (int b = CURVE_BITS - 1; b >= 0; --b)
+    for (int b = BITS - 1; b >= 0; --b)
 #pragma unroll
         for (int i = 0; i < 3; ++i) k = (k << 1) | (((X[i] ^ t) >> b) & 1u);
     return k;
 }
 
+template <bool FINE>
 __global__ void __launch_bounds__(256) curve_keys_kernel(const float4* __restrict__ pos, int n,
                                                        const float* __restrict__ bnd, int nb,
-                                                       unsigned* __restrict__ key, int* __restrict__ idx)
+                                                       typename Curve<FINE>::Key* __restrict__ key,
+                                                       int* __restrict__ idx)
 {
+    constexpr int BITS = Curve<FINE>::BITS;
     __shared__ float box[6];
     if (threadIdx.x < 192) {  // six warps, one component each
         const int c = threadIdx.x >> 5;
@@ -201,23 +213,33 @@ __global__ void __launch_bounds__(256) curve_keys_kernel(const float4* __restric
     if (i >= n) return;
     const float4 p = pos[i];
     const float ext = fmaxf(-box[3] - box[0], fmaxf(-box[4] - box[1], -box[5] - box[2]));
-    const float s = ext > 0.f && isfinite(ext) ? (float)(1 << CURVE_BITS) / ext : 0.f;
+    const float s = ext > 0.f && isfinite(ext) ? (float)(1 << BITS) / ext : 0.f;
     auto cell = [&](float x, float lo) {
         const float f = (x - lo) * s;  // a non-finite coordinate goes to cell 0
-        return f > 0.f ? min((unsigned)fminf(f, 1e6f), (1u << CURVE_BITS) - 1u) : 0u;
+        return f > 0.f ? min((unsigned)fminf(f, 4e6f), (1u << BITS) - 1u) : 0u;
     };
-    key[i] = hilbert_key(cell(p.x, box[0]), cell(p.y, box[1]), cell(p.z, box[2]));
+    key[i] = hilbert_key<FINE>(cell(p.x, box[0]), cell(p.y, box[1]), cell(p.z, box[2]));
     idx[i] = i;
 }
 
-bool curve_layout(int64_t n, Carve& cv, CurveWs& w)
+template <bool FINE>
+static cudaError_t curve_sort(void* ws, size_t& bytes, const void* key, void* key2, const int* idx, int* perm, int n,
+                              cudaStream_t st)
 {
-    const bool ok = cub::DeviceRadixSort::SortPairs(nullptr, w.cub_bytes, (const unsigned*)nullptr, (unsigned*)nullptr,
-                                                    (const int*)nullptr, (int*)nullptr, (int)n, 0,
-                                                    3 * CURVE_BITS) == cudaSuccess;
+    using Key = typename Curve<FINE>::Key;
+    return cub::DeviceRadixSort::SortPairs(ws, bytes, static_cast<const Key*>(key), static_cast<Key*>(key2), idx, perm,
+                                           n, 0, 3 * Curve<FINE>::BITS, st);
+}
+
+bool curve_layout(int64_t n, Carve& cv, CurveWs& w, bool fine)
+{
+    const bool ok = (fine ? curve_sort<true> : curve_sort<false>)(nullptr, w.cub_bytes, nullptr, nullptr, nullptr,
+                                                                  nullptr, (int)n, nullptr) == cudaSuccess;
+    const size_t key_bytes = fine ? sizeof(Curve<true>::Key) : sizeof(Curve<false>::Key);
+    w.fine = fine;
     w.bnd = cv.take(CURVE_BND_BLOCKS * 6 * sizeof(float));
-    w.key = cv.take((size_t)n * 4);
-    w.key2 = cv.take((size_t)n * 4);
+    w.key = cv.take((size_t)n * key_bytes);
+    w.key2 = cv.take((size_t)n * key_bytes);
     w.idx = cv.take((size_t)n * 4);
     w.perm = cv.take((size_t)n * 4);
     w.cub = cv.take(w.cub_bytes);
@@ -227,17 +249,20 @@ bool curve_layout(int64_t n, Carve& cv, CurveWs& w)
 cudaError_t run_curve_sort(const CurveWs& w, char* ws, const float4* pos, int n, cudaStream_t st)
 {
     float* bnd = reinterpret_cast<float*>(ws + w.bnd);
-    unsigned* key = reinterpret_cast<unsigned*>(ws + w.key);
-    unsigned* key2 = reinterpret_cast<unsigned*>(ws + w.key2);
     int* idx = reinterpret_cast<int*>(ws + w.idx);
     int* perm = reinterpret_cast<int*>(ws + w.perm);
     const int nb = std::min(CURVE_BND_BLOCKS, (n + 255) / 256);
     trace_launch(2);
     curve_bounds_kernel<<<nb, 256, 0, st>>>(pos, n, bnd);
-    curve_keys_kernel<<<(n + 255) / 256, 256, 0, st>>>(pos, n, bnd, nb, key, idx);
+    if (w.fine)
+        curve_keys_kernel<true><<<(n + 255) / 256, 256, 0, st>>>(
+            pos, n, bnd, nb, reinterpret_cast<Curve<true>::Key*>(ws + w.key), idx);
+    else
+        curve_keys_kernel<false><<<(n + 255) / 256, 256, 0, st>>>(
+            pos, n, bnd, nb, reinterpret_cast<Curve<false>::Key*>(ws + w.key), idx);
     size_t bytes = w.cub_bytes;
-    const cudaError_t e =
-        cub::DeviceRadixSort::SortPairs(ws + w.cub, bytes, key, key2, idx, perm, n, 0, 3 * CURVE_BITS, st);
+    const cudaError_t e = (w.fine ? curve_sort<true> : curve_sort<false>)(ws + w.cub, bytes, ws + w.key, ws + w.key2,
+                                                                         idx, perm, n, st);
     return e != cudaSuccess ? e : cudaGetLastError();
 }
 

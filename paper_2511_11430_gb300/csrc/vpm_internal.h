@@ -39,11 +39,12 @@ int* dev_err_ptr();          // device error word of the current device
 int sweep_blocks(bool grad, bool comp, bool stretch, int kind = 0);  // resident sweep blocks (current device)
 int adjoint_blocks(bool comp);
 
-// Workspace of the curve order of n particles (offsets).
+// Workspace of the curve order of n particles (offsets).  fine: 21 bits an axis instead of 8.
 struct CurveWs {
     size_t bnd = 0, key = 0, key2 = 0, idx = 0, perm = 0, cub = 0, cub_bytes = 0;
+    bool fine = false;
 };
-bool curve_layout(int64_t n, Carve& cv, CurveWs& w);  // false: the sort's scratch size could not be had
+bool curve_layout(int64_t n, Carve& cv, CurveWs& w, bool fine = false);  // false: the sort's scratch size could not be had
 // Hilbert-curve order of n particles: sorted position -> index in ws + w.perm.
 cudaError_t run_curve_sort(const CurveWs& w, char* ws, const float4* pos, int n, cudaStream_t st);
 

@@ -1474,7 +1474,7 @@ cudaError_t tree_rhs_layout(long long n, long long m, TreeRhsWs& r)
     r.nut = cv.take((size_t)n * sizeof(float));
     r.snut = cv.take((size_t)n * sizeof(float));
     r.box = cv.take(pse_box_bytes(n));
-    if (!curve_layout(n, cv, r.curve)) return cudaErrorUnknown;
+    if (!curve_layout(n, cv, r.curve, true)) return cudaErrorUnknown;
     r.bytes = cv.off;
     return cudaSuccess;
 }

@@ -77,3 +77,41 @@ def test_adjoint(api):
     assert rel_l2(dx[:, idx].double().cpu().numpy().T, rx) <= 1e-5
     assert rel_l2(dG[:, idx].double().cpu().numpy().T, rG) <= 1e-5
     assert api.device_error() == 0
+
+
+def _rhs_tree(api, w):
+    P, S, a, b = (to_dev(x) for x in (w.pos, w.strength, w.seg_a, w.seg_b))
+    prm = api.Params(sigma=w.sigma, nu=w.nu, c_v=w.c_v, seg_core=w.seg_core, u_inf=w.u_inf)
+    ws = api.Workspace("cuda")
+    run = lambda: api.rhs_tree(P, S, a, b, prm, theta=0.5, order=4, ws=ws)
+    out = run()
+    t = []
+    for _ in range(3):
+        e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        torch.cuda.synchronize()
+        e0.record()
+        run()
+        e1.record()
+        torch.cuda.synchronize()
+        t.append(e0.elapsed_time(e1))
+    return out, min(t)
+
+
+def test_tree_exchange_with_strays(api):
+    """The treecode's exchange takes the particles in curve order.  Three of them a thousand metres off must not
+    leave the rest in a few of the curve's cells: in no order every tile reaches every particle, and the call took
+    seven times as long.  (The tree itself differs with the strays, so the times are only of one size.)"""
+    n = 600_000
+    (_, dG, _), t0 = _rhs_tree(api, _wake(n, 0.0, "multirotor"))
+    w = _wake(n, 1000.0, "multirotor")
+    (_, dGs, nut), t1 = _rhs_tree(api, w)
+    assert t1 < 4.0 * t0, (t0, t1)
+    # the exchange itself, at sampled particles: what nu adds to dGamma/dt
+    P, S, a, b = (to_dev(x) for x in (w.pos, w.strength, w.seg_a, w.seg_b))
+    prm = lambda nu: api.Params(sigma=w.sigma, nu=nu, c_v=0.0, seg_core=w.seg_core, u_inf=w.u_inf)
+    big = 1.0  # so that the exchange outweighs the stretching, whose difference cancels but for rounding
+    d = api.rhs_tree(P, S, a, b, prm(big))[1] - api.rhs_tree(P, S, a, b, prm(0.0))[1]
+    idx = synth.sample_targets(5, n, 200)
+    ref = oracle.pse_at(w.pos, w.strength, np.zeros(n), w.sigma, big, idx)
+    assert rel_l2(d[:, idx].double().cpu().numpy().T, ref) <= 1e-5
+    assert api.device_error() == 0
