@@ -99,8 +99,8 @@ cudaError_t run_sweep(const SweepPlan& p, char* ws, const float* tgt, const floa
 cudaError_t run_pse(const SweepPlan& p, char* ws, const float* pos, const float* str, const float* nu_t, int n,
                     float sigma, float nu, float* dGdt, cudaStream_t st);
 
-// The same over n particles in the order pos, str, nu_t have; particle i's term goes to dGdt
-// element perm[i] (perm null: i).  box: room for the tile boxes (pse_box_bytes).
+// The same over n particles given in curve order; particle i's term goes to dGdt element
+// perm[i].  box: room for the tile boxes and those of groups of tiles (pse_box_bytes).
 size_t pse_box_bytes(int64_t n);
 cudaError_t run_pse_sorted(const float4* pos, const float4* str, const float* nu_t, const int* perm, float4* box, int n,
                            float sigma, float nu, float* dGdt, cudaStream_t st);

@@ -814,6 +814,11 @@ __global__ void __launch_bounds__(256) epilogue_kernel(const EpiArgs E)
 // ---------------------------------------------------------------------------
 constexpr int PSE_T = 512;
 constexpr int PSE_W = PSE_T / 32;
+// FAN: particles in curve order, where 32 consecutive tiles are compact too: their common box is
+// tested first, and the tiles of the few in reach.  Every block looks at every box, which with the
+// tiles' alone is quadratic in the count (treecode right-hand side, 4,000,000 of the BVI wake
+// 104.1 and 97.8 ms, 8,000,000 of the two-rotor wake 493 and 469 ms).
+constexpr int PSE_FAN = 32;
 
 __device__ __forceinline__ void pse_pair(float4 pi, float4 gi, float base, float4 pj, float4 gj, float ntj,
                                          float inv2s2, float cut2, float& ax, float& ay, float& az)
@@ -829,6 +834,7 @@ __device__ __forceinline__ void pse_pair(float4 pi, float4 gi, float base, float
     }
 }
 
+template <bool FAN>
 __global__ void __launch_bounds__(PSE_T) pse_kernel(const float4* __restrict__ pos, const float4* __restrict__ str,
                                                     const float* __restrict__ nu_t, int n,
                                                     const float4* __restrict__ box, int ntiles, float inv2s2,
@@ -854,39 +860,54 @@ __global__ void __launch_bounds__(PSE_T) pse_kernel(const float4* __restrict__ p
     // warp w takes the 32 sources w mod 4 of the tiles in reach whose number is w / 4 (mod PSE_W / 4)
     const int word = warp & 3, slot = warp >> 2;
     int met = 0;  // tiles in reach so far
-    for (int tb = 0, r = 0; tb < ntiles; tb += 32 * PSE_W, r ^= 1) {
+    auto visit = [&](int tile) {
+        if ((met++ & (PSE_W / 4 - 1)) != slot) return;
+        const int j = tile * SRC_TILE + 32 * word + lane;
+        // stage the sources; one at least 7 sigma from both of the warp's target boxes
+        // reaches none of its targets and is left out (warp-uniformly, by ballot)
+        __syncwarp();
+        bool kp = false;
+        if (j < n) {
+            const float4 pq = pos[j];
+            sp[lane] = pq;
+            sg[lane] = str[j];
+            snt[warp][lane] = nu_t ? nu_t[j] : 0.f;
+            const float4 pt = make_float4(pq.x, pq.y, pq.z, 0.f);
+            kp = boxes_near(wbox[warp], pt, pt, cut2);
+        }
+        unsigned m = __ballot_sync(0xffffffffu, kp);
+        __syncwarp();
+        for (; m; m &= m - 1) {
+            const int q = __ffs(m) - 1;
+            const float4 pj = sp[q], gj = sg[q];
+            const float ntj = snt[warp][q];
+            pse_pair(p0, g0, base0, pj, gj, ntj, inv2s2, cut2, a0x, a0y, a0z);
+            pse_pair(p1, g1, base1, pj, gj, ntj, inv2s2, cut2, a1x, a1y, a1z);
+        }
+    };
+    // one box a thread and round: of the tiles, or of PSE_FAN tiles each, which follow the tiles' boxes
+    const int nboxes = FAN ? (ntiles + PSE_FAN - 1) / PSE_FAN : ntiles;
+    const float4* outer = FAN ? box + 2 * (size_t)ntiles : box;
+    for (int tb = 0, r = 0; tb < nboxes; tb += PSE_T, r ^= 1) {
         const int tt = tb + 32 * warp + lane;
-        const bool near = tt < ntiles && boxes_near(wbox[warp], box[2 * tt], box[2 * tt + 1], cut2);
+        const bool near = tt < nboxes && boxes_near(wbox[warp], outer[2 * tt], outer[2 * tt + 1], cut2);
         const unsigned mine = __ballot_sync(0xffffffffu, near);
         if (lane == 0) found[r][warp] = mine;
         if (!__syncthreads_or((int)mine)) continue;
 #pragma unroll 1
         for (int w = 0; w < PSE_W; ++w)
-        for (unsigned mask = found[r][w]; mask; mask &= mask - 1, ++met) {
-            if ((met & (PSE_W / 4 - 1)) != slot) continue;
-            const int j = (tb + 32 * w + __ffs(mask) - 1) * SRC_TILE + 32 * word + lane;
-            // stage the sources; one at least 7 sigma from both of the warp's target boxes
-            // reaches none of its targets and is left out (warp-uniformly, by ballot)
-            __syncwarp();
-            bool kp = false;
-            if (j < n) {
-                const float4 pq = pos[j];
-                sp[lane] = pq;
-                sg[lane] = str[j];
-                snt[warp][lane] = nu_t ? nu_t[j] : 0.f;
-                const float4 pt = make_float4(pq.x, pq.y, pq.z, 0.f);
-                kp = boxes_near(wbox[warp], pt, pt, cut2);
+            for (unsigned mask = found[r][w]; mask; mask &= mask - 1) {
+                const int k = tb + 32 * w + __ffs(mask) - 1;
+                if constexpr (FAN) {
+                    const int t = k * PSE_FAN + lane;
+                    unsigned in = __ballot_sync(
+                        0xffffffffu, t < ntiles && boxes_near(wbox[warp], box[2 * (size_t)t], box[2 * (size_t)t + 1], cut2));
+#pragma unroll 1
+                    for (; in; in &= in - 1) visit(k * PSE_FAN + __ffs(in) - 1);
+                } else {
+                    visit(k);
+                }
             }
-            unsigned m = __ballot_sync(0xffffffffu, kp);
-            __syncwarp();
-            for (; m; m &= m - 1) {
-                const int q = __ffs(m) - 1;
-                const float4 pj = sp[q], gj = sg[q];
-                const float ntj = snt[warp][q];
-                pse_pair(p0, g0, base0, pj, gj, ntj, inv2s2, cut2, a0x, a0y, a0z);
-                pse_pair(p1, g1, base1, pj, gj, ntj, inv2s2, cut2, a1x, a1y, a1z);
-            }
-        }
     }
     // the warps' sums in a fixed order, one thread per target
     __syncthreads();
@@ -930,6 +951,31 @@ __global__ void __launch_bounds__(SRC_TILE) tile_box_kernel(const float4* __rest
             for (int c = 0; c < 6; ++c) v[c] = fminf(v[c], sb[w][c]);
         box[2 * blockIdx.x] = make_float4(v[0], v[1], v[2], 0.f);
         box[2 * blockIdx.x + 1] = make_float4(-v[3], -v[4], -v[5], 0.f);
+    }
+}
+
+// Boxes of PSE_FAN tiles each, behind the ntiles tile boxes; a warp per box.
+__global__ void __launch_bounds__(256) fan_box_kernel(float4* __restrict__ box, int ntiles)
+{
+    const int k = (blockIdx.x * 256 + threadIdx.x) >> 5, lane = threadIdx.x & 31, t = k * PSE_FAN + lane;
+    static_assert(PSE_FAN == 32, "a tile per lane");
+    if (k * PSE_FAN >= ntiles) return;
+    float lo[3] = {INFINITY, INFINITY, INFINITY}, hi[3] = {-INFINITY, -INFINITY, -INFINITY};
+    if (t < ntiles) {
+        const float4 a = box[2 * (size_t)t], b = box[2 * (size_t)t + 1];
+        lo[0] = a.x, lo[1] = a.y, lo[2] = a.z, hi[0] = b.x, hi[1] = b.y, hi[2] = b.z;
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            lo[c] = fminf(lo[c], __shfl_xor_sync(0xffffffffu, lo[c], o));
+            hi[c] = fmaxf(hi[c], __shfl_xor_sync(0xffffffffu, hi[c], o));
+        }
+    if (lane == 0) {
+        float4* out = box + 2 * ((size_t)ntiles + k);
+        out[0] = make_float4(lo[0], lo[1], lo[2], 0.f);
+        out[1] = make_float4(hi[0], hi[1], hi[2], 0.f);
     }
 }
 
@@ -1293,7 +1339,7 @@ cudaError_t run_sweep(const SweepPlan& p, char* ws, const float* tgt, const floa
 }
 
 static cudaError_t launch_pse(const float4* pos, const float4* str, const float* nu_t, const int* perm,
-                              const float4* box, int n, float sigma, float nu, float* dGdt, cudaStream_t st)
+                              const float4* box, bool fan, int n, float sigma, float nu, float* dGdt, cudaStream_t st)
 {
     const double s = sigma;
     const float inv2s2 = (float)(0.5 / (s * s));
@@ -1301,19 +1347,25 @@ static cudaError_t launch_pse(const float4* pos, const float4* str, const float*
     // (2/sigma^2) (2 pi sigma^2)^(-3/2)
     const float pref = (float)(2.0 / (s * s) * pow(2.0 * 3.14159265358979323846 * s * s, -1.5));
     TraceScope ts(VPM_TRACE_PSE, st);
-    pse_kernel<<<(n + 63) / 64, PSE_T, 0, st>>>(pos, str, nu_t, n, box, (n + SRC_TILE - 1) / SRC_TILE, inv2s2, cut2, nu,
-                                                pref, perm, dGdt);
+    (fan ? pse_kernel<true> : pse_kernel<false>)<<<(n + 63) / 64, PSE_T, 0, st>>>(
+        pos, str, nu_t, n, box, (n + SRC_TILE - 1) / SRC_TILE, inv2s2, cut2, nu, pref, perm, dGdt);
     return cudaGetLastError();
 }
 
-size_t pse_box_bytes(int64_t n) { return (size_t)((n + SRC_TILE - 1) / SRC_TILE) * 32; }
+size_t pse_box_bytes(int64_t n)
+{
+    const size_t tiles = (size_t)((n + SRC_TILE - 1) / SRC_TILE);
+    return (tiles + (tiles + PSE_FAN - 1) / PSE_FAN) * 32;
+}
 
 cudaError_t run_pse_sorted(const float4* pos, const float4* str, const float* nu_t, const int* perm, float4* box, int n,
                            float sigma, float nu, float* dGdt, cudaStream_t st)
 {
-    trace_launch();
-    tile_box_kernel<<<(n + SRC_TILE - 1) / SRC_TILE, SRC_TILE, 0, st>>>(pos, n, box);
-    return launch_pse(pos, str, nu_t, perm, box, n, sigma, nu, dGdt, st);
+    const int tiles = (n + SRC_TILE - 1) / SRC_TILE;
+    trace_launch(2);
+    tile_box_kernel<<<tiles, SRC_TILE, 0, st>>>(pos, n, box);
+    fan_box_kernel<<<((tiles + PSE_FAN - 1) / PSE_FAN + 7) / 8, 256, 0, st>>>(box, tiles);
+    return launch_pse(pos, str, nu_t, perm, box, true, n, sigma, nu, dGdt, st);
 }
 
 cudaError_t run_pse(const SweepPlan& p, char* ws, const float* pos, const float* str, const float* nu_t, int n,
@@ -1325,11 +1377,12 @@ cudaError_t run_pse(const SweepPlan& p, char* ws, const float* pos, const float*
     // the exchange takes the particles in the caller's order (filaments give its targets
     // tighter boxes than the curve does: 162 against 747 us at 100,000 particles with one
     // warp per 64 targets)
-    if (p.sort)
-        return run_pse_sorted(pos4, str4, nu_t, nullptr, reinterpret_cast<float4*>(ws + p.off_obox), n, sigma, nu, dGdt,
-                              st);
-    return launch_pse(pos4, str4, nu_t, nullptr, reinterpret_cast<const float4*>(ws + p.off_pbox), n, sigma, nu, dGdt,
-                      st);
+    float4* box = reinterpret_cast<float4*>(ws + (p.sort ? p.off_obox : p.off_pbox));
+    if (p.sort) {
+        trace_launch();
+        tile_box_kernel<<<(n + SRC_TILE - 1) / SRC_TILE, SRC_TILE, 0, st>>>(pos4, n, box);
+    }
+    return launch_pse(pos4, str4, nu_t, nullptr, box, false, n, sigma, nu, dGdt, st);
 }
 
 }  // namespace vpm

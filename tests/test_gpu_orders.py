@@ -115,3 +115,19 @@ def test_tree_exchange_with_strays(api):
     ref = oracle.pse_at(w.pos, w.strength, np.zeros(n), w.sigma, big, idx)
     assert rel_l2(d[:, idx].double().cpu().numpy().T, ref) <= 1e-5
     assert api.device_error() == 0
+
+
+@pytest.mark.parametrize("n", [65, 128, 129, 4_096, 4_097, 65_537])
+def test_tree_exchange_at_the_edges_of_tiles_and_groups(api, n):
+    """Tiles of 128 particles, groups of 32 tiles; a cloud about a core size apart, so that every size has pairs
+    within the exchange's 7 core sizes."""
+    sigma = n ** (-1.0 / 3.0)
+    pos, G = synth.random_cloud(3, n, box=1.0, sigma=sigma)
+    P, S = to_dev(pos), to_dev(G)
+    none = torch.empty((0, 4), dtype=torch.float32, device="cuda")
+    prm = lambda nu: api.Params(sigma=sigma, nu=nu, c_v=0.0)
+    d = api.rhs_tree(P, S, none, none, prm(1.0))[1] - api.rhs_tree(P, S, none, none, prm(0.0))[1]
+    idx = np.unique(np.concatenate([[0, n - 1], synth.sample_targets(5, n, min(n, 200))]))
+    ref = oracle.pse_at(pos, G, np.zeros(n), sigma, 1.0, idx)
+    assert rel_l2(d[:, idx].double().cpu().numpy().T, ref) <= 1e-5
+    assert api.device_error() == 0
