@@ -117,6 +117,10 @@ vpm_status vpm_device_error(int* code);
  *   VPM_OP_TREE:      n_src particles (vpm_tree_induce)
  *   VPM_OP_RHS_TREE, VPM_OP_STEP_TREE: n_src particles, m_seg segments
  *   VPM_OP_STAGE:     n_src particles, m_seg segments (vpm_rk3_stage)
+ * Never less for larger counts: a workspace for the largest counts of a program serves
+ * all of its calls.  (From 2^26 units of 1,024 targets by 128 sources on, 2,965,000
+ * particles on themselves, direct sums run without the tensor cores and their size
+ * holds 3 GB that only smaller calls use.)
  * `flags` as passed to the operation.  Host-only; does not launch. */
 vpm_status vpm_workspace_size(int op, int64_t n_src, int64_t n_tgt, int64_t m_seg, int flags, size_t* bytes);
 

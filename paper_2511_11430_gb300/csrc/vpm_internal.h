@@ -67,7 +67,7 @@ struct SweepPlan {
     CurveWs curve{};
     size_t off_spos = 0, off_sstr = 0, off_obox = 0;
     size_t off_ftile = 0, off_fmask = 0, off_fcnt = 0, off_nlist = 0, off_noff = 0, off_flist = 0, off_foff = 0,
-           off_part_f = 0, off_part_n = 0;
+           off_part_f = 0;
 };
 
 // Plans a particle + segment sweep onto `n_tgt` targets from a workspace carve: the

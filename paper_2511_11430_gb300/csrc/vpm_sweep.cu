@@ -1084,10 +1084,11 @@ SweepPlan plan_sweep(int64_t n_tgt, int64_t n_src, int64_t m_seg, bool grad, boo
     p.SP = (int)((n_src + SRC_TILE - 1) / SRC_TILE);
     p.SS = (int)((m_seg + SRC_TILE - 1) / SRC_TILE);
     const long long units_p = (long long)p.TT * p.SP;
-    const bool far_size =
-        allow_far && (n_tgt == n_src && grad ? n_src >= FAR_SORT_MIN
-                                             : units_p >= (grad ? FAR_MIN_UNITS_GRAD : FAR_MIN_UNITS_VEL));
-    p.far = far_size && units_p <= FAR_MAX_UNITS;
+    // The workspace must not shrink as a count grows (a caller may hold one for the largest counts it
+    // will have), so what the far sweep needs is reserved by the units alone, also where it is not used:
+    // particles onto themselves below FAR_SORT_MIN, and beyond FAR_MAX_UNITS.
+    const bool reserve = allow_far && units_p >= (grad ? FAR_MIN_UNITS_GRAD : FAR_MIN_UNITS_VEL);
+    p.far = reserve && units_p <= FAR_MAX_UNITS && !(n_tgt == n_src && grad && n_src < FAR_SORT_MIN);
     // particle tiles and segment tiles: one stream-K plan (and launch) each
     auto plan = [&](StreamK& sk, int kind, int np, int ns) {
         const bool teams = kind == SWEEP_SMALL || kind == SWEEP_SEG_SMALL;
@@ -1121,13 +1122,17 @@ SweepPlan plan_sweep(int64_t n_tgt, int64_t n_src, int64_t m_seg, bool grad, boo
     p.off_ssrc = cv.take((size_t)p.SS * SRC_TILE * S_F4 * 16);
     p.off_sbox = cv.take((size_t)p.SS * 2 * 16);
     const size_t rows = (size_t)(comp ? 2 : 1) * p.ncomp;
-    if (!p.far && p.sk.np + p.sk.ns > 0) p.off_part = cv.take((size_t)(p.sk.TT + p.sk.B) * rows * tgt_k * sizeof(float));
+    size_t part = p.sk.np + p.sk.ns > 0 ? (size_t)(p.sk.TT + p.sk.B) * rows * tgt_k * sizeof(float) : 0;
+    if (reserve) {  // one buffer for the particle launch's sums in either form
+        p.B_near = sweep_blocks(grad, comp, p.stretch, SWEEP_NEAR);
+        part = std::max(part, (size_t)(p.TT * FAR_GROUPS + p.B_near * Ring<SWEEP_NEAR>::TEAMS) * rows * FAR_GROUP * sizeof(float));
+    }
+    if (part > 0) p.off_part = cv.take(part);
     if (p.sks.ns > 0) p.off_part_s = cv.take((size_t)(p.sks.TT + p.sks.B) * rows * tgt_s * sizeof(float));
     // Units on the tensor cores
-    if (far_size) {
+    if (reserve) {
         p.KY = (p.SP + FAR_KCH - 1) / FAR_KCH;
-        const long long units = p.far ? units_p : FAR_MAX_UNITS;  // beyond the limit: keep the size monotone
-        p.B_near = sweep_blocks(grad, comp, p.stretch, SWEEP_NEAR);
+        const long long units = std::min(units_p, FAR_MAX_UNITS);
         p.B_far = (int)std::min<long long>(std::max(sm_count(), 1), units);
         const size_t rows_f = (size_t)(comp ? 2 : 1) * (grad ? 14 : 3);
         p.off_ftile = cv.take((size_t)p.SP * far_tile_bytes(grad));
@@ -1138,15 +1143,13 @@ SweepPlan plan_sweep(int64_t n_tgt, int64_t n_src, int64_t m_seg, bool grad, boo
         p.off_flist = cv.take((size_t)units * sizeof(uint2));
         p.off_foff = cv.take(((size_t)p.TT * p.KY + 1) * sizeof(uint2));
         p.off_part_f = cv.take((size_t)(p.TT + p.B_far) * rows_f * TGT_TILE * sizeof(float));
-        constexpr int teams = Ring<SWEEP_NEAR>::TEAMS;
-        p.off_part_n = cv.take((size_t)(p.TT * FAR_GROUPS + p.B_near * teams) * rows * FAR_GROUP * sizeof(float));
-        if (n_tgt == n_src) {
-            const size_t n = (size_t)n_src;
-            const bool sortable = curve_layout(n_src, cv, p.curve);
-            p.sort = p.far && grad && sortable;
+        if (grad) {  // particles onto themselves, which fewer targets or sources may be
+            const size_t n = (size_t)std::min(n_src, n_tgt);
+            const bool sortable = curve_layout((int64_t)n, cv, p.curve);
+            p.sort = p.far && n_tgt == n_src && sortable;
             p.off_spos = cv.take(n * 16);
             p.off_sstr = cv.take(n * 16);
-            p.off_obox = cv.take((size_t)p.SP * 2 * 16);
+            p.off_obox = cv.take((n + SRC_TILE - 1) / SRC_TILE * 2 * 16);
         }
     }
     p.bytes = cv.off;
@@ -1277,7 +1280,6 @@ cudaError_t run_sweep(const SweepPlan& p, char* ws, const float* tgt, const floa
                                              : std::min(A.sk.B, sweep_blocks(p.grad, p.comp, p.stretch, k));
             if (k == SWEEP_NEAR) {
                 A.ul = uln;
-                A.part = reinterpret_cast<float*>(ws + p.off_part_n);
                 FarArgs F;
                 F.tgt = A.tgt;
                 F.n_tgt = p.n_tgt;
@@ -1309,7 +1311,7 @@ cudaError_t run_sweep(const SweepPlan& p, char* ws, const float* tgt, const floa
     }
     EpiArgs E;
     E.sk = p.sk;
-    E.part = p.far ? reinterpret_cast<const float*>(ws + p.off_part_n) : part;
+    E.part = part;
     E.sks = p.sks;
     E.part_s = part_s;
     E.tgt = p.kind == SWEEP_SMALL ? Ring<SWEEP_SMALL>::TGT : TGT_TILE;
