@@ -296,11 +296,17 @@ constexpr int SWEEP_KINDS = 5;
 // half tiles 64 sources): a small problem then reaches every SM, and a few targets or a few
 // waves of units leave less idle.  (2,000 particles and 640 segments: 42 units of
 // 1,024 x 128, 73 us.)
-// Units (1,024 targets x 128 sources) below which teams sweep the particle tiles, and the
+// Units (1,024 targets x 128 sources) below which teams sweep the particle tiles; above, whole
+// blocks, which share a source tile among 16 warps, unless the targets fill few tiles, whose last
+// is mostly empty (u and grad u of a wake's particles by vpm_induce_noalloc, teams and whole
+// blocks: 16,000 of the hover wake 363 and 357 us, 30,000 1,111 and 1,036 us; of the BVI wake 382
+// and 412, 1,182 and 1,235 us.  Teams alone took up to 9% longer than the whole blocks that they
+// had replaced on the hover wake).  Likewise for the
 // segment tiles (whose loop pays more for the folds after half tiles: 5,120 segments onto
 // 100,000 particles 1.25 ms with whole blocks and tiles, 1.43 ms with teams; onto 20,000, 5.3
 // units a block, 317 and 324 us).
-constexpr long long SMALL_MAX_UNITS = 16384, SEG_SMALL_MAX_UNITS = 512;
+constexpr long long SMALL_MAX_UNITS = 4096, SEG_SMALL_MAX_UNITS = 512;
+constexpr int SMALL_FEW_TILES = 8;
 // Segment tiles up to which a small problem sweeps them, one segment at a time, with its
 // particle tiles.
 constexpr int MIXED_MAX_TILES = 8;
@@ -1110,8 +1116,8 @@ SweepPlan plan_sweep(int64_t n_tgt, int64_t n_src, int64_t m_seg, bool grad, boo
     // A small problem with few segments sweeps both kinds of tile in one launch; otherwise the
     // segment tiles have a launch of their own, where closed rings are packed by corner.
     const long long units_s = (long long)p.TT * p.SS;
-    p.mixed = p.SP > 0 && p.SS > 0 && p.SS <= MIXED_MAX_TILES && !p.far && units_p < SMALL_MAX_UNITS;
-    p.kind = units_p < SMALL_MAX_UNITS ? SWEEP_SMALL : SWEEP_PARTICLES;
+    p.kind = units_p < SMALL_MAX_UNITS || p.TT < SMALL_FEW_TILES ? SWEEP_SMALL : SWEEP_PARTICLES;
+    p.mixed = p.SP > 0 && p.SS > 0 && p.SS <= MIXED_MAX_TILES && !p.far && p.kind == SWEEP_SMALL;
     p.kind_s = units_s < SEG_SMALL_MAX_UNITS ? SWEEP_SEG_SMALL : SWEEP_SEGMENTS;
     plan(p.sk, p.kind, p.SP, p.mixed ? p.SS : 0);
     plan(p.sks, p.kind_s, 0, p.mixed ? 0 : p.SS);
