@@ -21,7 +21,7 @@
 // strengths of neighbours; here they are unrelated and g_k may be far smaller: dL/dx 1e-5
 // off at |g| = 1e-3 |Gamma| and 1e-2 off at 1e-6.)  A problem large
 // enough for the tensor cores (FAR_MIN_UNITS_GRAD) runs so; adjoint_kernel
-// takes the smaller ones (1,280 points, 110,000 particles: 223 and 196 us).
+// takes the smaller ones (1,280 points, 100,000 particles: 267 and 210 us).
 #include <algorithm>
 #include <math.h>
 
@@ -360,8 +360,8 @@ namespace {
 // With the control points as sources of strength g, the adjoint is what the particle sweep
 // computes at the particles: dL/dGamma = u (K r x g = K g x (x_j - y_k)) and dL/dx = J^T Gamma.
 // A problem large enough for the tensor cores takes that path (200,000 particles and 1,280
-// control points: 407 us by adjoint_kernel, 291 us so); a smaller one adjoint_kernel, which
-// accumulates 6 rows instead of 14 (60,000 particles: 170 against 185 us).
+// control points: 440 us by adjoint_kernel, 288 us so); a smaller one adjoint_kernel, which
+// accumulates 6 rows instead of 14 (60,000 particles: 199 against 230 us).
 struct SweepAdj {
     SweepPlan p;
     size_t off_g, bytes;

@@ -26,7 +26,7 @@
 // (32 TMEM columns, the accumulators take the other 32 of a tile's 64); the last warp of a
 // group to store its rows issues the chunk's twelve MMAs while the others go on.
 // 400,000 particles onto themselves, compensated: 161 ms by the pair sweep alone, 70 ms so
-// (2.3e12 pairs/s); 100,000: 10.4 and 5.2 ms.
+// (2.3e12 pairs/s); 100,000: 10.2 and 5.0 ms.
 //
 // A (target group, tile) pair takes this path when the tile's radius is at most FAR_TAU of
 // its centre's distance to the group's boxes and every pair is at least 7 sigma apart (the
@@ -53,14 +53,16 @@ constexpr int FAR_COST_FIRST = 3;                // cost of a far unit's first g
 constexpr float FAR_TAU = 0.5f;
 // (1,024-target, 128-source) units from which the far sweep is used: below, packing and
 // listing (about 40 us) cost more than it saves.  Velocity only, 1,280 control points:
-// 100,000 sources (1,564 units) 176 us without it and 185 us with it, 150,000 (2,344 units)
-// 240 and 229 us.  With the gradient, the adjoint of 1,280 control points at 60,000 particles
-// (590 units) 185 and 235 us, at 110,000 (1,080 units) 223 and 196 us.
+// 100,000 sources (1,564 units) 146 us without it and 171 us with it, 160,000 (2,500 units)
+// 205 and 212, 200,000 (3,126 units) 245 and 241, 300,000 337 and 310 us.  With the gradient, the
+// adjoint of 1,280 control points at 60,000 particles (590 units) 199 and 230 us, at 100,000
+// (980 units) 267 and 210 us.  As many targets as sources, in tensors of their own, depend on the
+// order that they come in (20,000, u and grad u: hover wake 559 and 613 us, BVI wake 597 and 430).
 constexpr long long FAR_MIN_UNITS_VEL = 2048, FAR_MIN_UNITS_GRAD = 900;
 constexpr long long FAR_MAX_UNITS = 1LL << 26;   // ... and to which (the unit lists take up to 44 bytes each)
 // Particles onto themselves: smallest count put in curve order and swept this way (right-hand
-// side of the BVI wake: 16,000 particles 819 us without and 744 us with it, 12,000 particles
-// 611 and 638 us; hover wake 679 and 690 us, 488 and 572 us).
+// side, without and with it: BVI wake 12,000 particles 617 and 628 us, 16,000 822 and 743 us, 20,000
+// 1,050 and 876 us; hover wake 571 and 586, 724 and 727, 945 and 864 us).
 constexpr int FAR_SORT_MIN = 16384;
 // Coordinates up to which |x - y|^2 stays finite in FP32.  Beyond, a pair contributes nothing
 // in the pair sweep (1/r of an infinite r^2), which takes the groups and tiles concerned.

@@ -23,8 +23,8 @@
 // targets there are.  Far from a warp's 64 targets (the tile's bounding box more
 // than 7 sigma from both of the warp's two target boxes) the blob kernel equals
 // the point-vortex kernel to FP32 precision, so far tiles run the 1/r^3 form with
-// one rsqrt; near tiles evaluate the regularised kernel for the sources within 7 sigma of
-// the warp's boxes.  In larger problems the tiles that are far and compact run on the
+// one rsqrt; near tiles evaluate the regularised kernel for the sources within 7 sigma (of
+// the warp's boxes with stretching, of a thread's targets without).  In larger problems the tiles that are far and compact run on the
 // tensor cores instead (vpm_far.cuh), over particles in curve order.  Each tile's sums start from zero and are folded into a
 // per-thread running sum kept in shared memory: a compensated (hi, lo) pair with
 // Knuth's two-sum, or a plain sum, so long source lists keep a tile-sized error.
@@ -814,7 +814,8 @@ __global__ void __launch_bounds__(256) epilogue_kernel(const EpiArgs E)
 // them, 32 sources at a time: a warp stages its sources (positions, strengths, nu_t) in its
 // own slice of shared memory with coalesced loads, then every lane sums over them; the
 // warps' sums are added in a fixed order.  (One warp per 64 particles left most SMs idle
-// below 50,000 particles: 71 us for 2,000 and 86 us for 20,000; eight warps 30 and 33 us.)  v_i Gamma_j - v_j Gamma_i is formed from two
+// below 50,000 particles: 71 us for 2,000 and 86 us for 20,000; sixteen warps 21 and 34 us.)
+// v_i Gamma_j - v_j Gamma_i is formed from two
 // rounded products so that the i == j term is exactly zero; pairs beyond 7 sigma
 // get exp(-r^2/2s^2) < 3e-11 and are skipped.
 // ---------------------------------------------------------------------------
@@ -1152,6 +1153,9 @@ SweepPlan plan_sweep(int64_t n_tgt, int64_t n_src, int64_t m_seg, bool grad, boo
         if (grad) {  // particles onto themselves, which fewer targets or sources may be
             const size_t n = (size_t)std::min(n_src, n_tgt);
             const bool sortable = curve_layout((int64_t)n, cv, p.curve);
+            // With the gradient only: the velocity alone costs so little that the sort does not pay on a
+            // wake in its own order (17,000 of the BVI wake 294 us without and 329 us with it, 60,000
+            // 1,582 and 1,679; of the hover wake 296 and 314, 1,771 and 1,716 us).
             p.sort = p.far && n_tgt == n_src && sortable;
             p.off_spos = cv.take(n * 16);
             p.off_sstr = cv.take(n * 16);
@@ -1382,9 +1386,8 @@ cudaError_t run_pse(const SweepPlan& p, char* ws, const float* pos, const float*
     if (n == 0) return cudaSuccess;
     const float4* pos4 = reinterpret_cast<const float4*>(pos);
     const float4* str4 = reinterpret_cast<const float4*>(str);
-    // the exchange takes the particles in the caller's order (filaments give its targets
-    // tighter boxes than the curve does: 162 against 747 us at 100,000 particles with one
-    // warp per 64 targets)
+    // the exchange takes the particles in the caller's order, which needs no sorted copy of nu_t
+    // (100,000 particles of the hover wake: 164 us, in curve order 158; 20,000: 34 and 44)
     float4* box = reinterpret_cast<float4*>(ws + (p.sort ? p.off_obox : p.off_pbox));
     if (p.sort) {
         trace_launch();
