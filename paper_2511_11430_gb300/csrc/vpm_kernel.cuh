@@ -131,7 +131,7 @@ __device__ __forceinline__ void near_kh(float r2, const NearConst& nc, float& K,
 // branches of near_kh cost the sum of the forms present in a warp, on each packed lane
 // in turn.  Its one branch leaves out the rest where neither of a thread's targets is within
 // 7 sigma, as in most of the near tiles of particles in no order (100,000 onto points of their
-// own, u and grad u: 17.1 ms with near_kh, 25.5 ms without the branch, 14.6 with it).
+// own, u and grad u: 17.1 ms with near_kh, 25.5 ms without the branch, 15.0 with it).
 __device__ __forceinline__ void near_kh2(f2 r2, const NearConst& nc, f2& K, f2& h)
 {
     const f2 rs = rsqrt2_approx(r2);

@@ -495,12 +495,19 @@ __global__ void __launch_bounds__(SWEEP_TPB, 1) sweep_kernel(const SweepArgs A)
         // stretching from the tile's sums afterwards.  Near particle tiles accumulate the
         // stretching pair by pair (it cancels there) with the strengths loaded for them.
         const int ti0 = t * R::TGT + (warp % R::WARPS) * 64 + lane, ti1 = ti0 + 32;
-        // Near sources summed in a row.  In curve order a target's neighbours fill whole tiles, and the
-        // rounding of their sums grows with the run, where in the caller's order they were spread over
-        // many tiles; halved, it is below what it was there (20,011-particle hover wake, error of nu_t:
-        // 8.9e-7 in the caller's order, 9.8e-7 in curve order and whole tiles, 7.1e-7 in halves; 886
-        // and 884 us a right-hand side).
-        constexpr int NEAR_RUN = LIST && COMP && GRAD ? SRC_TILE / 2 : R::UNIT;
+        // Near sources summed in a row before the fold.  In curve order a target's neighbours fill whole
+        // tiles, and the rounding of their sums grows with the run, where in the caller's order they were
+        // spread over many tiles; in halves it is below what it was there (20,011-particle hover wake,
+        // error of nu_t: 8.9e-7 in the caller's order, 9.8e-7 in curve order and whole tiles, 7.1e-7 in
+        // halves; 886 and 884 us a right-hand side; plain sums 9.6e-7, 1.13e-6, 7.8e-7).  Without
+        // stretching near and far sources come mixed and there are fewer rows to fold: 32 (velocity at
+        // 1,280 points of the BVI wake, 250,007 particles: 8.4e-8 with whole tiles, 4.7e-8; its adjoint
+        // dL/dx 2.0e-7 with halves, 1.6e-7; the times within 1%).  Teams' half tiles are short enough.
+        constexpr int NEAR_RUN = KIND == SWEEP_PARTICLES ? R::UNIT
+                                 : !GRAD                 ? 32
+                                 : !LIST                 ? R::UNIT
+                                 : !STRETCH && COMP      ? 32
+                                                         : SRC_TILE / 2;
         if (LIST || (!R::SEG && k < sk.np)) {
             const int cnt = min(R::UNIT, A.n_src - k * R::UNIT);  // (the last half tile may be empty)
             const float4 tlo = src[R::BOX], thi = src[R::BOX + 1];
@@ -539,7 +546,7 @@ __global__ void __launch_bounds__(SWEEP_TPB, 1) sweep_kernel(const SweepArgs A)
                         finish_tile<GRAD, STRETCH>(acc, tf, A.tstr, ti0, ti1, A.n_tgt);
                     }
                     particle_subset<GRAD, true, true>(acc, src, keep, 0, NEAR_RUN / 32, false, cnt, X, Y, Z, A.nc, own);
-                    if (NEAR_RUN < SRC_TILE && (keep[2] | keep[3])) {
+                    if (LIST && (keep[2] | keep[3])) {
                         fold_acc();
                         acc.zero();
                         particle_subset<GRAD, true, true>(acc, src, keep, NEAR_RUN / 32, SRC_TILE / 32, false, cnt, X, Y, Z, A.nc,

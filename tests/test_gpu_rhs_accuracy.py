@@ -11,21 +11,23 @@ torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("n", [20_011, 24_001])
-def test_eddy_viscosity_as_in_the_callers_order(n):
+@pytest.mark.parametrize("n,compensated,bound", [(20_011, True, 9.3e-7), (24_001, True, 9.3e-7), (20_011, False, 1.0e-6)])
+def test_eddy_viscosity_as_in_the_callers_order(n, compensated, bound):
     """nu_t amplifies the gradient's rounding most.  Summed in the caller's order (the pair sweep without curve
-    order) its error on this wake is 8.8e-7 to 8.9e-7; 5% are allowed for another order of the rounding."""
+    order) its error on this wake is 8.8e-7 to 8.9e-7, in plain sums 9.6e-7; 5% are allowed for another order of
+    the rounding."""
     if not torch.cuda.is_available():
         pytest.skip("no CUDA device")
     from paper_2511_11430_gb300 import api, build
 
     build.build()
     w = synth.hover(seed=1, n=n)
-    prm = api.Params(sigma=w.sigma, nu=w.nu, c_v=w.c_v, seg_core=w.seg_core, u_inf=w.u_inf)
+    prm = api.Params(sigma=w.sigma, nu=w.nu, c_v=w.c_v, seg_core=w.seg_core, u_inf=w.u_inf, compensated=compensated,
+                     classic=not compensated)
     _, _, nut = api.rhs(to_dev(w.pos), to_dev(w.strength), to_dev(w.seg_a), to_dev(w.seg_b), prm)
     idx = np.arange(0, n, 2)
     _, J = oracle.p2p(w.pos, w.strength, w.pos[idx], w.sigma)
     _, Js = oracle.segments(w.seg_a, w.seg_b, w.pos[idx], w.seg_core, 2)
     ref = oracle.vreman(J + Js, w.sigma, w.c_v)
-    assert rel_l2(nut[idx].double().cpu().numpy(), ref) <= 9.3e-7
+    assert rel_l2(nut[idx].double().cpu().numpy(), ref) <= bound
     assert api.device_error() == 0
