@@ -38,12 +38,12 @@ FLOPS_P2P = 54   # u + grad u, far-field operation tree, FFMA = 2 flops
 FLOPS_SEG = 120  # Vatistas segment u + grad u, same counting convention
 L2_FLUSH_BYTES = 256 << 20
 TOL = {"compensated": 2e-6, "plain": 1e-4, "nu_t": {"compensated": 1e-5, "plain": 1e-3}}
-# DRAM bytes (read + write) of one particle sweep with gradient (the far_sweep_kernel and near
-# sweep_kernel launches), from one ncu capture per workload (profiles/far_sweep_kernel.md), keyed by
+# DRAM bytes (read + write) of one right-hand side's particle sweep with gradient: the far_sweep_kernel and
+# the near sweep_kernel launch of one ncu capture per workload (profiles/far_sweep_kernel.md), keyed by
 # (particles, segments); valid only while the kernel's sources hash to SWEEP_SRC_SHA256,
 # else the bench reports traffic null.
-SWEEP_TRAFFIC_BYTES = {(2_000_000, 7_680): 142_549_244_000 + 355_496_960}
-SWEEP_SRC_SHA256 = "554c12209b1a3bebcca23b4f0ce95552fb9362a866002d2d20a1288ac8c463fe"
+SWEEP_TRAFFIC_BYTES = {(2_000_000, 7_680): 423_572_677_888 + 292_882_688 + 2_550_501_632 + 274_675_200}
+SWEEP_SRC_SHA256 = "cfef8c3791b00b202f1dd58555a79036edcd3d985112190b804d1e35ee7015cc"
 SWEEP_SRC = ["paper_2511_11430_gb300/csrc/vpm_sweep.cu", "paper_2511_11430_gb300/csrc/vpm_kernel.cuh",
              "paper_2511_11430_gb300/csrc/vpm_far.cu", "paper_2511_11430_gb300/csrc/vpm_far.cuh",
              "paper_2511_11430_gb300/csrc/vpm_common.cuh"]
@@ -577,6 +577,15 @@ def error_report(gpu, ref, idx_u, idx_r):
     return rep
 
 
+def tensor_peak():
+    """The measured dense bf16 GEMM rate of this card where a record of it lies beside this file."""
+    try:
+        with open(os.path.join(ROOT, "MEASURED_PEAKS.json")) as fh:
+            return float(json.load(fh)["bf16_tflops"]), "measured dense bf16 GEMM (burst)"
+    except (OSError, KeyError, ValueError):
+        return 1900.0, "dense bf16 GEMM, an earlier measurement (burst)"
+
+
 def roofline(tr, n, m, sms, clk):
     from paper_2511_11430_gb300 import _lib
 
@@ -588,22 +597,28 @@ def roofline(tr, n, m, sms, clk):
     # a small problem sweeps its segment tiles in the particle launch (no segment launch)
     flops_launch = FLOPS_P2P * n * (n - 1) + (FLOPS_SEG * n * m if not ns_ else 0)
     achieved = flops_launch / (avg_ms * 1e-3) / 1e12
-    kernel = ("far_sweep_kernel<grad, compensated> + sweep_kernel<grad, compensated, stretch, near>" if n >= 16384
+    far = 16384 <= n < 2_965_000  # the far tiles on the tensor cores
+    kernel = ("far_sweep_kernel<grad, compensated> + sweep_kernel<grad, compensated, stretch, near>" if far
               else "sweep_kernel<grad, compensated, stretch, teams>")
-    roof = {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "TFLOP/s", "frac": achieved / peak,
-            "traffic": sweep_traffic(n, m), "kernel": kernel,
+    bound, basis = "alu", f"{sms} SMs x 128 FP32 lanes x 2 (FFMA) x {sm_max:.0f} MHz max SM clock (derived)"
+    fp32, note = peak, "flops of the direct pair form"
+    if far:
+        bound, peak, basis = "tensor", *tensor_peak()
+        note += ("; a pair's weight takes 7 FP32 operations, a rsqrt and an FP16 split beside its products, so "
+                 "issue slots and the FMA and XU pipes bound the sweep; frac_fp32 is of the FP32 peak, which holds "
+                 "for the pair loop alone")
+    roof = {"bound": bound, "achieved": achieved, "peak": peak, "unit": "TFLOP/s", "frac": achieved / peak,
+            "frac_fp32": achieved / fp32, "traffic": sweep_traffic(n, m), "kernel": kernel,
             "launches": nl, "avg_launch_ms": avg_ms, "flops_per_launch": flops_launch,
-            "peak_basis": f"{sms} SMs x 128 FP32 lanes x 2 (FFMA) x {sm_max:.0f} MHz max SM clock (derived)",
-            "note": "flops of the direct pair form; the far tiles' products run on the tensor cores, so the rate can "
-                    "pass the FP32 peak; what bounds them is issue slots and the FMA pipe"}
+            "peak_basis": basis, "note": note}
     if ns_ and m:
         seg_avg = seg_ms / ns_
         seg_t = FLOPS_SEG * n * m / (seg_avg * 1e-3) / 1e12
         roof["segment_launch"] = {"kernel": "sweep_kernel<grad, compensated, stretch, segment tiles>",
                                   "launches": ns_, "avg_launch_ms": seg_avg, "flops_per_launch": FLOPS_SEG * n * m,
-                                  "achieved": seg_t, "frac": seg_t / peak}
+                                  "achieved": seg_t, "frac": seg_t / fp32}
     if clk and clk.get("sm_mhz"):
-        roof["frac_at_measured_clock"] = achieved / (sms * 128 * 2 * clk["sm_mhz"] * 1e6 / 1e12)
+        roof["frac_fp32_at_measured_clock"] = achieved / (sms * 128 * 2 * clk["sm_mhz"] * 1e6 / 1e12)
     return roof
 
 

@@ -45,11 +45,11 @@ constexpr unsigned FAR_ALL = (1u << FAR_GROUPS) - 1u;
 // Cost in the pair sweep of a warp's tile within 7 sigma, against one of a tile beyond.
 constexpr int NEAR_COST = 3;
 constexpr int FAR_COST_FIRST = 3;                // cost of a far unit's first group, against one of each further
-// Acceptance ratio.  The error does not depend on it where it was measured (0.2 to 0.6: u
-// 1.31e-7 to 1.34e-7, grad u 1.83e-7 throughout on the 100,000-particle hover wake, whose
-// error comes from the near pairs), since every pair is evaluated at any ratio; beyond 0.5
-// the weights (up to 31 there) and the cancellation in t grow and little time is gained
-// (hover wake, 100,000: 7.20 ms at 0.2, 6.23 at 0.33, 5.88 at 0.5, 5.63 at 0.6).
+// Acceptance ratio.  The error hardly depends on it, since every pair is evaluated at any ratio
+// (right-hand side of the 100,000-particle hover wake at 0.33, 0.4 and 0.5: dx/dt 1.08e-7, 1.09e-7 and
+// 1.13e-7, nu_t 9.96e-7, 9.96e-7 and 9.97e-7, with the near tiles' sums folded once a tile); beyond 0.5
+// the weights (up to 31 there) and the cancellation in t grow and little time is gained (the same
+// call 7.05, 6.94 and 6.82 ms; u and grad u alone 5.88 ms at 0.5 and 5.63 at 0.6 in an earlier form).
 constexpr float FAR_TAU = 0.5f;
 // (1,024-target, 128-source) units from which the far sweep is used: below, packing and
 // listing (about 40 us) cost more than it saves.  Velocity only, 1,280 control points:
